@@ -433,10 +433,11 @@ vox_status vox_generate_noalloc(const vox_segment *d_segs, int64_t n, vox_dims d
 /*
  * Launch tuning (process-wide, every device). The outputs do not depend on it:
  * only how the work is spread. Chosen by measurement (the Python autotuner).
- *   run_len       voxels per thread run in the list/atomic generation kernel:
- *                 16, 32 or 64 (0 = default: 32; 64-bit lists take 64 as 32);
- *                 longer runs pay the run's entry less often, shorter runs keep
- *                 more threads busy on small inputs
+ *   run_len       voxels per thread run in the per-voxel atomic volume kernel
+ *                 (with or without a list in the same launch): 16, 32 or 64 (0 =
+ *                 default: 32; 64-bit lists take 64 as 32); longer runs pay the
+ *                 run's entry less often, shorter runs keep more threads busy on
+ *                 small inputs
  *   volume_path   VOX_VOLUME_AUTO (bricks when the workspace allows; pieces
  *                 beyond the workspace by per-voxel atomics), VOX_VOLUME_ATOMIC
  *                 (always per-voxel atomics: each thread merges the bits of
@@ -445,18 +446,12 @@ vox_status vox_generate_noalloc(const vox_segment *d_segs, int64_t n, vox_dims d
  *                 alone also merged across the warp: at every step the lanes
  *                 holding equal words (__match_any_sync) OR their bits together
  *                 (__reduce_or_sync) and one lane issues the reduction)
- *   ctas_per_sm   persistent CTAs per SM for the generation and brick kernels
- *                 (0 = the occupancy maximum; larger values are capped there)
- *   list_runs     a list alone (no volume in the same launch, or the volume
- *                 by bricks): 0 = a thread's run of run_len voxels continues
- *                 into the next segments (best when segments share one length
- *                 that run_len divides or that divides run_len); 1 = 32-bit
- *                 lists only: runs end at segment ends (best for short segments
- *                 of varying length); 2 = warp slices: each warp writes 1056
- *                 consecutive voxels (lanes' runs of 33) in list order into
- *                 shared memory and stores them with one TMA bulk copy, taking
- *                 slices from a global work counter (32- and 64-bit lists; best
- *                 for long segments); other values are 0
+ *   ctas_per_sm   persistent CTAs per SM for the atomic and brick kernels, and the
+ *                 unit in which a list's grid is sized (0 = the occupancy maximum;
+ *                 larger values are capped there)
+ *   list_runs     0, 1 or 2 (other values are 0): no effect. A list alone (no
+ *                 volume in the same launch, or the volume by bricks) has one
+ *                 kernel, whatever the segment lengths
  * vox_set_tuning(NULL) restores the defaults. Not to be changed while calls
  * are being issued from other host threads.
  */

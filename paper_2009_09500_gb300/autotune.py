@@ -7,12 +7,11 @@ and caches it in a JSON file keyed by the GPU name and a workload class, so a
 later run with a similar workload reuses it without measuring.
 
 Tuned knobs (see include/vox.h, vox_tuning):
-  run_len      voxels per thread run in the generation kernel (16, 32 or 64)
+  run_len      voxels per thread run in the atomic volume kernel (16, 32 or 64)
   volume_path  bricks when the workspace allows (auto), per-voxel atomics, or
                per-voxel atomics merged across the warp
   ctas_per_sm  persistent CTAs per SM (0 = occupancy maximum, or fewer)
-  list_runs    a list alone: thread runs across segment ends (0), 32-bit runs
-               cut at them (1), or warp slices stored by TMA bulk copies (2)
+  list_runs    no effect any more (a list alone has one kernel)
 """
 
 from __future__ import annotations

@@ -28,7 +28,6 @@ constexpr size_t kWsAlign = 256;
 constexpr int64_t kMaxDim = int64_t(1) << 21;
 constexpr int64_t kMinPerCta = 2048;          // smallest voxel range given to one CTA
 constexpr int64_t kDefaultWaitNs = 500000000;  // 0.5 s bound on every in-kernel wait
-constexpr size_t kListCounterOffset = 128;    // k_list's chunk counter, in the workspace's ticket region
 
 std::atomic<int64_t> g_stall_tile{-1};
 std::atomic<int64_t> g_wait_ns{kDefaultWaitNs};
@@ -375,17 +374,6 @@ vox_status launch_gen_t(const GenParams &p, cudaStream_t stream)
     if constexpr ((OUT & kOutList64) != 0) {
         if (current_tuning().run_len == 16) return launch_gen_r<16, OUT, LIN64>(p, stream);
         return launch_gen_r<32, OUT, LIN64>(p, stream);
-    } else if constexpr (OUT == kOutList32) {
-        // a 32-bit list alone may cut its runs at segment ends (list_runs = 1)
-        const vox_tuning tu = current_tuning();
-        if (tu.list_runs == 1 && p.scene_of == nullptr) {
-            if (tu.run_len == 16) return launch_gen_r<16, OUT | kOutSegRuns, LIN64>(p, stream);
-            if (tu.run_len == 64) return launch_gen_r<64, OUT | kOutSegRuns, LIN64>(p, stream);
-            return launch_gen_r<32, OUT | kOutSegRuns, LIN64>(p, stream);
-        }
-        if (tu.run_len == 16) return launch_gen_r<16, OUT, LIN64>(p, stream);
-        if (tu.run_len == 64) return launch_gen_r<64, OUT, LIN64>(p, stream);
-        return launch_gen_r<32, OUT, LIN64>(p, stream);
     } else if constexpr (OUT == kOutMask) {
         // the volume alone: per-lane word runs, or merged across the warp too
         const vox_tuning tu = current_tuning();
@@ -404,29 +392,26 @@ vox_status launch_gen_t(const GenParams &p, cudaStream_t stream)
     }
 }
 
-// The list alone by warp slices (k_list): persistent grid, the chunk counter in
-// the workspace's ticket region reset first.
+// The list alone (k_list): the grid from the capacity, the voxels per warp from the total
+// that the scan found, so that a capacity far above it costs only CTAs with smaller chunks.
 template <typename PackT>
 vox_status launch_list(const vox_segment *segs, int64_t n, void *list, int64_t capacity, void *ws, int32_t *status,
                        cudaStream_t stream)
 {
-    const WsLayout L = ws_layout(n);
-    char *base = static_cast<char *>(ws);
     ListParams p;
     p.segs = reinterpret_cast<const int32_t *>(segs);
     p.n = n;
-    p.offsets = reinterpret_cast<const int64_t *>(base + L.offsets);
+    p.offsets = reinterpret_cast<const int64_t *>(static_cast<char *>(ws) + ws_layout(n).offsets);
     p.list = list;
     p.capacity = capacity;
     p.status = status;
-    p.counter = reinterpret_cast<uint32_t *>(base + kListCounterOffset);
     auto kernel = k_list<PackT>;
-    const size_t smem = sizeof(ListWarpSmem<PackT>) * kListWarps;
-    if (vox_status e = allow_smem(reinterpret_cast<const void *>(kernel), smem)) return e;
-    const int grid = grid_ctas(reinterpret_cast<const void *>(kernel), kListThreads, smem);
-    if (grid <= 0) return VOX_ERR_CUDA;
-    if (cudaMemsetAsync(p.counter, 0, sizeof(uint32_t), stream) != cudaSuccess) return VOX_ERR_CUDA;
-    kernel<<<static_cast<unsigned>(grid), kListThreads, smem, stream>>>(p);
+    const int64_t resident = grid_ctas(reinterpret_cast<const void *>(kernel), kListThreads, 0);
+    if (resident <= 0) return VOX_ERR_CUDA;
+    const int64_t per_warp = capacity / (resident * kListWarps);
+    const int64_t rounds = std::max<int64_t>(1, (per_warp + kListChunkMax - 1) / kListChunkMax);
+    const int64_t grid = std::min<int64_t>(resident * rounds, int64_t(1) << 30);
+    kernel<<<static_cast<unsigned>(grid), kListThreads, 0, stream>>>(p);
     return cudaGetLastError() == cudaSuccess ? VOX_OK : VOX_ERR_CUDA;
 }
 
@@ -460,18 +445,14 @@ vox_status launch_generate(const vox_segment *segs, int64_t n, vox_dims dims, vo
     // batched volumes may differ in size: 64-bit bit indices cover them all
     const bool lin64 = scene_of != nullptr || volume_bits(dims) > (uint64_t(1) << 32);
     const bool bm = flags & VOX_OUT_BITMASK;
-    if (!bm && current_tuning().list_runs == 2) {  // a list alone by warp slices
+    if (!bm) {  // a list alone
         if (flags & VOX_OUT_LIST32) return launch_list<uint32_t>(segs, n, list, capacity, ws, status, stream);
-        if (flags & VOX_OUT_LIST64) return launch_list<uint64_t>(segs, n, list, capacity, ws, status, stream);
+        return launch_list<uint64_t>(segs, n, list, capacity, ws, status, stream);
     }
-    if (flags & VOX_OUT_LIST32) {
-        return bm ? launch_gen_t<kOutList32 | kOutMask, false>(p, stream) : launch_gen_t<kOutList32, false>(p, stream);
-    }
-    if (flags & VOX_OUT_LIST64) {
-        if (!bm) return launch_gen_t<kOutList64, false>(p, stream);
+    if (flags & VOX_OUT_LIST32) return launch_gen_t<kOutList32 | kOutMask, false>(p, stream);
+    if (flags & VOX_OUT_LIST64)
         return lin64 ? launch_gen_t<kOutList64 | kOutMask, true>(p, stream)
                      : launch_gen_t<kOutList64 | kOutMask, false>(p, stream);
-    }
     return lin64 ? launch_gen_t<kOutMask, true>(p, stream) : launch_gen_t<kOutMask, false>(p, stream);
 }
 

@@ -1,36 +1,35 @@
-// vox_list.cuh -- the packed voxel list by warp slices and TMA bulk stores (sm_103a).
+// vox_list.cuh -- the packed voxel list, one row of 32 voxels per warp and step (sm_103a).
 //
 // The list of Fig. 3 / Section 4 (every voxel of every segment, in segment order,
-// at offsets[s] + k) is written by warps that own slices of kListSlice = 32 x 33
-// consecutive global voxel ids. Lane l of a warp takes the run of kListRun = 33
-// voxels starting at slice position 33 l and steps through it with the exact
-// carry recurrence of Eq. (3) (vox_device.cuh), entering its first segment by one
-// division per minor axis and the following ones at k = 0. The voxels go to a
-// per-warp stage in shared memory in their final (linear) order: with an odd run
-// length, lane l's u-th voxel sits at word 33 l + u, bank (l + u) mod 32, so the
-// 32 lanes' stores never collide (64-bit voxels: two lanes per bank pair, the
-// minimum for 256 bytes). The finished slice leaves with one TMA bulk copy from
-// shared to global memory (cp.async.bulk), so the SM issues no load/store
-// instructions for the write-out and no CTA-wide barrier: each warp runs on its
-// own, taking chunks of slices from a global work counter (one atomic and one
-// search in the offsets per chunk; 1 to 16 slices per chunk, about eight chunks
-// per warp, so that short lists still spread evenly).
+// at offsets[s] + k). Voxel k does not depend on voxel k - 1 (Section 3), and with
+// a fixed-point slope it needs no division either, so lane l of a warp computes
+// voxel g + l of a row of 32 consecutive voxels outright and the row is stored
+// coalesced: no run per lane, no stage in shared memory, no transposition.
 //
-// A slice with few segment ends inside it (kListFlatMax at most, counted in the
-// staged window) is walked by the lanes in step over their runs: four voxels at
-// a time while no lane is within four voxels of its segment's or run's end (one
-// vote per four voxels), else one voxel, a voxel that ends its segment being
-// followed in place by the next segment's first voxel (entered at k = 0, no
-// division); the few lanes that cross a segment end hold the others up only for
-// that entry. A slice with many ends is walked part by part (one part per
-// segment), so that the lanes' entries happen together instead of one after
-// another.
+// Per axis the coordinate is the integer part of X0 + k T (mod 2^bits), with F
+// fraction bits and S = ceil(|d| 2^F / N):
+//   d >= 0:  X0 = S0 2^F + 2^(F-1),      T = S      floor(S0 + 1/2 + k S / 2^F)
+//   d <  0:  X0 = S0 2^F + 2^(F-1) - 1,  T = -S     floor(S0 + 1/2 - k S / 2^F - 2^-F)
+// The exact position S0 + 1/2 +- k |d| / N is a multiple of 1 / 2N, so its integer
+// part is unchanged by an error below 1 / 2N away from the side where a tie falls;
+// the error is below k 2^-F (plus 2^-F when d < 0), so F with (N + 1) 2^-F <= 1 / 2N
+// gives Eq. (3) with ties away from S, exactly:
+//   32-bit lists (edges <= 1024, N <= 1023): F = 22, one 32-bit word per axis;
+//   64-bit lists (N < 2^21): F = 43, one 64-bit word per axis.
+// The slopes are divided out once per staged segment (a lane per segment of the
+// window), not once per run of voxels.
 //
-// Segment records and offsets are staged per warp in windows of 32 segments
-// (plain coalesced loads into the warp's shared memory) and kept for the next
-// slice of the chunk while at least 16 of the window's segments lie ahead of
-// it; a slice that spans more segments is processed in several windows, each
-// lane keeping its stepping state across them.
+// What bounds it: HBM writes for 64-bit lists of long segments, instruction issue
+// for short ones (75 % of issue slots on 64-voxel segments; about 110 instructions a
+// row that holds segment starts, a row being 128 32-bit or 64 64-bit voxels).
+// Measured (GB300, list kernel alone), against runs of 33 voxels per lane stepped by
+// the carry recurrence into a shared stage (long segments) and 32-voxel thread runs
+// with a transposed stage (the rest):
+//   4M log-uniform segments in 4096^3, 64-bit, 2.07e9 voxels   2720 -> 2308 us
+//   1024 segments, 10^9 voxels, 64-bit                         1090 -> 1051 us
+//   1M log-uniform segments in 1000^3, 64-bit, 1.4e8 voxels     301 ->  208 us
+//   300,000 uniform segments in 256^3, 32-bit, 4.2e7 voxels      76 ->   54 us
+//   1M segments of 64 voxels, 32-bit, 6.7e7 voxels               78 ->   76 us
 #pragma once
 
 #include <cstdint>
@@ -42,15 +41,18 @@
 
 namespace vox {
 
-constexpr int kListRun = 33;                   // voxels per lane run (odd)
-constexpr int kListSlice = 32 * kListRun;      // voxels per warp slice (1056, a multiple of 4)
-constexpr int kListWarps = 4;                  // warps per CTA
+constexpr int kListWarps = 8;                  // warps per CTA
 constexpr int kListThreads = 32 * kListWarps;
-constexpr int kListWin = 32;                   // segments per staged window
-constexpr int kListChunkMax = 16;              // slices per fetch from the work counter, at most
-constexpr int kListChunksPerWarp = 8;          // chunks per warp aimed at (for balance)
-constexpr int kListFlatMax = 12;                // segment ends per slice up to which runs cross them in place
-static_assert(kListSlice % 4 == 0, "slices must keep 16-byte aligned list addresses");
+constexpr int kListCtas = 4;                   // CTAs per SM
+constexpr int kListWin = 32;                   // segments per staged window, one per lane
+// The list is cut into one chunk of consecutive voxels per warp of the grid. The grid
+// is sized from the capacity (launch_list): the resident CTAs as many times as keeps a
+// chunk within kListChunkMax. The CTAs beyond the
+// resident ones start in order as others end, so the warps at work at any moment
+// write one front of the list (see the figures at k_list).
+constexpr int kListChunkUnit = 128;            // chunks are multiples of a row
+constexpr int kListChunkMin = 256;             // voxels per warp at least
+constexpr int kListChunkMax = 6144;            // and at most
 
 struct ListParams {
     const int32_t *segs;     // [n][6]
@@ -59,17 +61,44 @@ struct ListParams {
     void *list;              // uint32 or uint64 list, 16-byte aligned
     int64_t capacity;
     int32_t *status;
-    uint32_t *counter;       // chunk counter, zeroed before the launch
 };
 
+// Fixed-point words of a list type: F fraction bits, integer parts on top.
+template <typename PackT>
+struct ListFix;
+
+template <>
+struct ListFix<uint32_t> {
+    static constexpr int F = 22;
+    // x | y << 10 | z << 20 from the top 10 bits of each word
+    static __device__ __forceinline__ uint32_t pack(uint32_t x, uint32_t y, uint32_t z)
+    {
+        return (x >> 22) | ((y >> 12) & 0x000ffc00u) | ((z >> 2) & 0x3ff00000u);
+    }
+};
+
+template <>
+struct ListFix<uint64_t> {
+    static constexpr int F = 43;
+    // x | y << 21 | z << 42 from the top 21 bits of each word, half by half
+    static __device__ __forceinline__ uint64_t pack(uint64_t x, uint64_t y, uint64_t z)
+    {
+        const uint32_t xh = static_cast<uint32_t>(x >> 32), yh = static_cast<uint32_t>(y >> 32),
+                       zh = static_cast<uint32_t>(z >> 32);
+        const uint32_t lo = (xh >> 11) | ((yh << 10) & 0xffe00000u);
+        const uint32_t hi = (yh >> 22) | ((zh >> 1) & 0x7ffffc00u);
+        return (static_cast<uint64_t>(hi) << 32) | lo;
+    }
+};
+
+// A window of segments as the lanes read it: field by field, so that lanes reading
+// different segments hit different banks.
 template <typename PackT>
 struct ListWarpSmem {
-    alignas(16) PackT stage[kListSlice];   // the slice's voxels in list order (bulk-copy source)
-    int64_t offs[kListWin + 1];            // offsets of the window's segments (+ the next)
-    int32_t recs[kListWin * 6];            // the window's segment records
+    PackT X0[3][kListWin];        // coordinates of voxel 0 (fixed point, half added)
+    PackT T[3][kListWin];         // per-voxel steps
+    int32_t rel[kListWin + 1];    // first voxel of each segment, relative to the chunk (+ the next)
 };
-static_assert(sizeof(ListWarpSmem<uint32_t>) % 16 == 0 && sizeof(ListWarpSmem<uint64_t>) % 16 == 0,
-              "per-warp regions keep the stage 16-byte aligned");
 
 // Largest s in [0, n) with offsets[s] <= g (offsets[0] <= g < offsets[n]): a
 // 32-ary search in which every lane probes one position per round; called by
@@ -89,27 +118,48 @@ __device__ __forceinline__ int64_t warp_find_segment(const int64_t *offsets, int
     return lo;
 }
 
-// Largest j in [0, cnt) with offs[j] <= r, given offs[0] <= r < offs[cnt], cnt <= 32.
-__device__ __forceinline__ int32_t find_in_window32(const int64_t *offs, int32_t cnt, int64_t r)
+__device__ __forceinline__ void prefetch_l1(const void *p)
 {
-    int32_t lo = 0;
-#pragma unroll
-    for (int32_t step = 16; step > 0; step >>= 1) {
-        const int32_t m = lo + step;
-        if (m < cnt && offs[m] <= r) lo = m;
-    }
-    return lo;
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
-template <typename PackT>
-__global__ void __launch_bounds__(kListThreads) k_list(ListParams p)
+__device__ __forceinline__ int4 list_quad(const uint32_t (&v)[4])
 {
-    extern __shared__ __align__(16) unsigned char list_smem_raw[];
+    return make_int4(static_cast<int>(v[0]), static_cast<int>(v[1]), static_cast<int>(v[2]), static_cast<int>(v[3]));
+}
+
+__device__ __forceinline__ int4 list_quad(const uint64_t (&v)[2])
+{
+    return make_int4(static_cast<int>(v[0]), static_cast<int>(v[0] >> 32), static_cast<int>(v[1]),
+                     static_cast<int>(v[1] >> 32));
+}
+
+// k t for a signed step count k given in two's complement (modulo the word).
+__device__ __forceinline__ uint32_t mul_signed(uint32_t k, uint32_t t) { return k * t; }
+__device__ __forceinline__ uint64_t mul_signed(uint32_t k, uint64_t t)
+{
+    return static_cast<uint64_t>(static_cast<int64_t>(static_cast<int32_t>(k))) * t;
+}
+
+// One chunk per warp, written front to back. What the chunks' order is worth: with
+// persistent warps taking every n_warps-th chunk the warps drift apart, and 2.07e9
+// 64-bit voxels take 2785 us; with CTAs started in order (or chunks from a global
+// counter) the writes stay one front and take 2308 us (7.2 TB/s). Chunks of 8192 /
+// 12288 voxels at most: 2353 / 2451 us; 2048: 3416 us (the search per chunk). Rows
+// collected in shared memory and stored by 4 KB bulk copies: 2421 us, and 88 instead
+// of 76 us on 64-voxel segments.
+template <typename PackT>
+__global__ void __launch_bounds__(kListThreads, kListCtas) k_list(ListParams p)
+{
+    using Fix = ListFix<PackT>;
+    constexpr int kVox = 16 / sizeof(PackT);  // consecutive voxels per lane and row: one 16-byte store
+    constexpr int kRow = 32 * kVox;
+    __shared__ ListWarpSmem<PackT> s_win[kListWarps];
     __shared__ int32_t s_go;
     __shared__ int64_t s_V;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    ListWarpSmem<PackT> &sm = reinterpret_cast<ListWarpSmem<PackT> *>(list_smem_raw)[warp];
+    ListWarpSmem<PackT> &sm = s_win[warp];
 
     // prologue decided by one thread so that the whole CTA agrees
     if (threadIdx.x == 0) {
@@ -126,178 +176,148 @@ __global__ void __launch_bounds__(kListThreads) k_list(ListParams p)
     if (!s_go) return;
     const int64_t V = s_V;
     PackT *const list = static_cast<PackT *>(p.list);
-    const int64_t n_slices = (V + kListSlice - 1) / kListSlice;
     const int64_t n_warps = static_cast<int64_t>(gridDim.x) * kListWarps;
-    const int64_t chunk_slices = max64(1, min64(kListChunkMax, n_slices / (n_warps * kListChunksPerWarp)));
-    const int64_t kChunk = chunk_slices * kListSlice;
-    bool pending = false;  // lane 0: a bulk store may still be reading this warp's stage
+    const int64_t per = ((V + n_warps - 1) / n_warps + kListChunkUnit - 1) & ~int64_t(kListChunkUnit - 1);
+    const int64_t chunk = max64(kListChunkMin, per);
+    const uint32_t le_mask = 0xffffffffu >> (31 - lane);  // this lane and those below
 
-    while (true) {
-        uint32_t c = 0;
-        if (lane == 0) c = atomicAdd(p.counter, 1u);
-        c = __shfl_sync(0xffffffffu, c, 0);
-        const int64_t g_begin = static_cast<int64_t>(c) * kChunk;
-        if (g_begin >= V) break;
-        const int64_t g_end = min64(g_begin + kChunk, V);
-        int64_t s = warp_find_segment(p.offsets, p.n, g_begin, lane);
-        int64_t ws_keep = -1;   // the staged window of the previous slice
-        int32_t wcnt_keep = 0;
-        for (int64_t g = g_begin; g < g_end; g += kListSlice) {
-            const int32_t len = static_cast<int32_t>(min64(kListSlice, g_end - g));
-            const int32_t my0 = kListRun * lane;
-            const int32_t rlen = max(0, min(kListRun, len - my0));
-            if (lane == 0 && pending) bulk_wait_read_all();  // the stage is free again
-            __syncwarp();
-
-            Stepper<PackT, uint32_t> st;
-            int32_t done = 0;
-            int64_t cur = -1;   // the segment being walked (-1: not found yet)
-            int32_t kin = 0;    // step at which to enter it
-            bool live = false;  // stepping state valid for cur
-            bool ended = false; // the last voxel written ended its segment
-            // keep the previous slice's window while 16 of its segments lie ahead
-            bool staged = ws_keep >= 0 && s >= ws_keep && s + kListWin / 2 <= ws_keep + wcnt_keep;
-            int64_t ws = staged ? ws_keep : s;  // first segment of the window
-            while (__any_sync(0xffffffffu, done < rlen)) {
-                const int32_t wcnt = staged ? wcnt_keep : static_cast<int32_t>(min64(kListWin, p.n - ws));
-                __syncwarp();  // every lane is done with the previous window
-                if (!staged) {
-                    const int64_t sj = ws + lane;
-                    if (lane < wcnt) {
-                        const int2 *r = reinterpret_cast<const int2 *>(p.segs + 6 * sj);
-                        const int2 a = __ldg(r), b = __ldg(r + 1), e = __ldg(r + 2);
-                        int32_t *d = sm.recs + 6 * lane;
-                        d[0] = a.x; d[1] = a.y; d[2] = b.x; d[3] = b.y; d[4] = e.x; d[5] = e.y;
-                    }
-                    if (lane <= wcnt) sm.offs[lane] = __ldg(p.offsets + sj);
-                    if (lane == 0 && wcnt == kListWin) sm.offs[kListWin] = __ldg(p.offsets + ws + kListWin);
-                }
-                __syncwarp();
-                // segment ends inside the slice that this window holds: with few, the
-                // lanes cross them in one loop over their runs (entering the next
-                // segment in place); with many, a loop per segment part keeps the
-                // entries together
-                const bool flat = __popc(__ballot_sync(0xffffffffu, lane >= 1 && lane <= wcnt && sm.offs[lane] > g &&
-                                                                         sm.offs[lane] < g + len)) <= kListFlatMax;
-                if (done < rlen && cur < 0) {  // the segment of the run's first voxel, if in this window
-                    const int64_t r = g + my0;
-                    if (r < sm.offs[wcnt]) {
-                        const int32_t j = find_in_window32(sm.offs, wcnt, r);
-                        cur = ws + j;
-                        kin = static_cast<int32_t>(r - sm.offs[j]);
-                    }
-                }
-                // the flat walk's votes need every lane: flat is the same for the whole warp
-                if (flat) {
-                    // the lanes walk in step: four voxels at once while no walking
-                    // lane is within four voxels of its segment's or run's end,
-                    // else one voxel, a segment end crossed in place
-                    bool go = cur >= 0 && done < rlen && cur < ws + wcnt;  // walks in this window
-                    if (go && !live) {
-                        st.enter(sm.recs + 6 * static_cast<int32_t>(cur - ws), kin, 0u, 0u);
-                        live = true;
-                    }
-                    int32_t left = go ? st.left : 0;  // voxels after this one in its segment
-                    int32_t u = done;
-                    while (__any_sync(0xffffffffu, go)) {
-                        if (__all_sync(0xffffffffu, !go || (left >= 4 && u + 4 <= rlen))) {
-                            if (go) {
+    const int64_t g0 = (static_cast<int64_t>(blockIdx.x) * kListWarps + warp) * chunk;
+    if (g0 < V) {
+        const int32_t len = static_cast<int32_t>(min64(chunk, V - g0));
+        PackT *const out = list + g0;
+        int64_t s = warp_find_segment(p.offsets, p.n, g0, lane);
+        int32_t pos = 0;  // positions are relative to g0
+        while (pos < len) {
+            // ---- the window: 32 segments from the one that holds `pos`
+            const int32_t wcnt = static_cast<int32_t>(min64(kListWin, p.n - s));
+            int32_t rel = 0x7fffffff;
+            __syncwarp();  // every lane is done with the previous window
+            if (lane < wcnt) {
+                int32_t r[6];
+                load_record(p.segs, s + lane, r);
+                rel = static_cast<int32_t>(__ldg(p.offsets + s + lane) - g0);
+                sm.rel[lane] = rel;
+                if (lane == wcnt - 1) sm.rel[wcnt] = static_cast<int32_t>(__ldg(p.offsets + s + wcnt) - g0);
+                const uint32_t N = static_cast<uint32_t>(max(abs(r[3] - r[0]), max(abs(r[4] - r[1]), abs(r[5] - r[2]))));
 #pragma unroll
-                                for (int v = 0; v < 4; ++v) {
-                                    sm.stage[my0 + u + v] = st.P;
-                                    st.template step<true, false>();
-                                }
-                                u += 4;
-                                left -= 4;
-                                ended = false;
-                                go = u < rlen;
-                            }
-                            continue;
-                        }
-                        if (go) {
-                            sm.stage[my0 + u] = st.P;
-                            ended = (left == 0);
-                            ++u;
-                            if (!ended) {
-                                --left;
-                                st.template step<true, false>();
-                                go = u < rlen;
-                            } else if (u == rlen) {  // the run ends with its segment
-                                go = false;
-                            } else {                 // the run goes on in the next segment
-                                ++cur;
-                                kin = 0;
-                                live = false;
-                                if (cur >= ws + wcnt) {  // ... which a later window holds
-                                    go = false;
-                                } else {
-                                    st.enter(sm.recs + 6 * static_cast<int32_t>(cur - ws), 0, 0u, 0u);
-                                    live = true;
-                                    left = st.left;
-                                }
-                            }
-                        }
-                    }
-                    done = u;
-                } else if (done < rlen) {
-                    PackT *o = sm.stage + my0 + done;
-                    while (cur >= 0 && done < rlen && cur < ws + wcnt) {
-                        if (!live) {
-                            st.enter(sm.recs + 6 * static_cast<int32_t>(cur - ws), kin, 0u, 0u);
-                            live = true;
-                        }
-                        const int32_t m = min(st.left + 1, rlen - done);
-                        ended = (m == st.left + 1);
-                        int32_t e = 0;
-                        for (; e + 4 <= m; e += 4) {
-#pragma unroll
-                            for (int v = 0; v < 4; ++v) {
-                                o[v] = st.P;
-                                st.template step<true, false>();
-                            }
-                            o += 4;
-                        }
-                        for (; e < m; ++e) {
-                            *o++ = st.P;
-                            st.template step<true, false>();
-                        }
-                        done += m;
-                        if (done < rlen) {  // the run goes on in the next segment
-                            ++cur;
-                            kin = 0;
-                            live = false;
-                        }
-                    }
-                }
-                ws_keep = ws;
-                wcnt_keep = wcnt;
-                staged = false;  // a further round stages the next window
-                if (__any_sync(0xffffffffu, done < rlen)) {
-                    ws += wcnt;
-                    if (wcnt == 0) break;  // unreachable for a consistent scan; keeps the loop finite
+                for (int a = 0; a < 3; ++a) {
+                    const int32_t d = r[3 + a] - r[a];
+                    const PackT A = static_cast<PackT>(abs(d));
+                    const PackT S = A == N ? PackT(1) << Fix::F  // the major axis, and minor ones as long
+                                           : ((A << Fix::F) + (N - 1u)) / N;
+                    sm.X0[a][lane] = (static_cast<PackT>(r[a]) << Fix::F) + (PackT(1) << (Fix::F - 1)) - (d < 0 ? 1 : 0);
+                    sm.T[a][lane] = d < 0 ? PackT(0) - S : S;
                 }
             }
-            // the next slice starts in the segment of this slice's last voxel, or
-            // the next one if that voxel ended its segment
-            const int last = (len - 1) / kListRun;
-            const int64_t cur_last = __shfl_sync(0xffffffffu, cur, last);
-            const bool ended_last = __shfl_sync(0xffffffffu, ended ? 1 : 0, last) != 0;
-            s = cur_last + (ended_last ? 1 : 0);
-
-            // write-out: the 16-byte part by one bulk copy, a ragged end (only at
-            // the end of the list) by plain stores
-            fence_proxy_async_smem();  // this lane's stage writes, visible to the bulk-copy unit
-            __syncwarp();
-            const uint32_t bytes = (static_cast<uint32_t>(len) * sizeof(PackT)) & ~15u;
-            if (lane == 0 && bytes) {
-                bulk_store_1d(list + g, sm.stage, bytes);
-                pending = true;
+            // the next 32 segments' records and offsets on their way to L1
+            if (s + 2 * kListWin <= p.n) {
+                if (lane < 24) prefetch_l1(p.segs + 6 * (s + kListWin) + 8 * lane);
+                else prefetch_l1(p.offsets + s + kListWin + 4 * (lane - 24));
             }
-            const int32_t tail0 = static_cast<int32_t>(bytes / sizeof(PackT));
-            for (int32_t e = tail0 + lane; e < len; e += 32) list[g + e] = sm.stage[e];
+            __syncwarp();
+            const int32_t wend = sm.rel[wcnt];
+            int32_t j = 0;  // the window's segment that holds pos
+            while (true) {
+                // a row needs the window to cover it; without that the window moves on
+                // to segment j, or (already there, or the list ends) 32 voxels are taken
+                const bool covered = pos + kRow <= min(wend, len);
+                if (!covered && j > 0 && wend < len) break;
+                // the segments that start in the row after its first voxel, by the first
+                // lane whose voxels all follow the start; two of them at one lane: short
+                // segments, 32 voxels at a time
+                const int32_t b = rel - pos;
+                const bool inside = b > 0 && b < kRow;
+                const uint32_t starts = __reduce_or_sync(0xffffffffu, inside ? 2u << ((b - 1) / kVox) : 0u);
+                if (covered && starts == 0u) {
+                    const int32_t e = sm.rel[j + 1];
+                    if (e - pos >= kRow) {
+                        // rows inside one segment
+                        const uint32_t k = static_cast<uint32_t>(pos + kVox * lane - sm.rel[j]);
+                        const PackT tx = sm.T[0][j], ty = sm.T[1][j], tz = sm.T[2][j];
+                        PackT x = sm.X0[0][j] + k * tx, y = sm.X0[1][j] + k * ty, z = sm.X0[2][j] + k * tz;
+                        const int32_t stop = min(e, len) - kRow;
+                        int4 *o = reinterpret_cast<int4 *>(out + pos) + lane;
+#pragma unroll 2
+                        for (; pos <= stop; pos += kRow) {
+                            PackT v[kVox];
+#pragma unroll
+                            for (int i = 0; i < kVox; ++i) {
+                                v[i] = Fix::pack(x, y, z);
+                                const uint32_t f = i + 1 < kVox ? 1u : static_cast<uint32_t>(kRow - kVox + 1);
+                                x += f * tx;
+                                y += f * ty;
+                                z += f * tz;
+                            }
+                            *o = list_quad(v);
+                            o += 32;
+                        }
+                        if (pos >= len) break;
+                        if (e <= pos) {
+                            ++j;
+                            if (j >= wcnt) break;
+                        }
+                        continue;
+                    }
+                }
+                // (a start among the last lane's voxels has no such lane)
+                const int32_t n_in = __popc(__ballot_sync(0xffffffffu, inside));
+                const int32_t n_last = __popc(__ballot_sync(0xffffffffu, inside && b > kRow - kVox));
+                if (covered && n_last <= 1 && __popc(starts) + n_last == n_in) {
+                    // a row with segment starts, at most one per lane
+                    const int32_t p0 = pos + kVox * lane;
+                    const int32_t jl = j + __popc(starts & le_mask);
+                    const int32_t c = sm.rel[jl + 1] - p0;  // this lane's voxels from c on are the next segment's
+                    const uint32_t k = static_cast<uint32_t>(p0 - sm.rel[jl]);
+                    const PackT tx = sm.T[0][jl], ty = sm.T[1][jl], tz = sm.T[2][jl];
+                    PackT x = sm.X0[0][jl] + k * tx, y = sm.X0[1][jl] + k * ty, z = sm.X0[2][jl] + k * tz;
+                    PackT v[kVox];
+#pragma unroll
+                    for (int i = 0; i < kVox; ++i) {
+                        v[i] = Fix::pack(x, y, z);
+                        x += tx;
+                        y += ty;
+                        z += tz;
+                    }
+                    if (c < kVox) {
+                        const uint32_t back = 0u - static_cast<uint32_t>(c - 1);  // voxel 1 is its step 1 - c
+                        const PackT ux = sm.T[0][jl + 1], uy = sm.T[1][jl + 1], uz = sm.T[2][jl + 1];
+                        x = sm.X0[0][jl + 1] + mul_signed(back, ux);
+                        y = sm.X0[1][jl + 1] + mul_signed(back, uy);
+                        z = sm.X0[2][jl + 1] + mul_signed(back, uz);
+#pragma unroll
+                        for (int i = 1; i < kVox; ++i) {
+                            if (i >= c) v[i] = Fix::pack(x, y, z);
+                            x += ux;
+                            y += uy;
+                            z += uz;
+                        }
+                    }
+                    reinterpret_cast<int4 *>(out + pos)[lane] = list_quad(v);
+                    pos += kRow;
+                    j += n_in;
+                } else {
+                    // 32 voxels, one per lane (the window covers them: 32 segments hold at
+                    // least 32 voxels): a bit for each start, and each lane counts the bits
+                    // up to its own position
+                    if (wend < len && pos + 32 > wend) break;
+                    const uint32_t bits = __reduce_or_sync(0xffffffffu, (b > 0 && b < 32) ? 1u << b : 0u);
+                    const int32_t jl = j + __popc(bits & le_mask);
+                    const uint32_t k = static_cast<uint32_t>(pos + lane - sm.rel[jl]);
+                    const PackT x = sm.X0[0][jl] + k * sm.T[0][jl], y = sm.X0[1][jl] + k * sm.T[1][jl],
+                                z = sm.X0[2][jl] + k * sm.T[2][jl];
+                    if (pos + lane < len) out[pos + lane] = Fix::pack(x, y, z);
+                    pos += 32;
+                    j += __popc(bits);
+                }
+                if (pos >= len) break;
+                if (sm.rel[j + 1] <= pos) {  // the next row starts a segment
+                    ++j;
+                    if (j >= wcnt) break;
+                }
+            }
+            s += j;
         }
     }
-    if (lane == 0 && pending) bulk_wait_all();  // copies complete before the CTA's memory goes
 }
 
 }  // namespace vox
