@@ -314,7 +314,7 @@ vox_status vox_generate_batched(const vox_segment *d_segs, int64_t n_total, cons
 
 /*
  * Batched volumes by bricks (the brick path of the single-scene volume, over
- * all scenes at once; one counter replica, bricks merged by plain stores):
+ * all scenes at once; bricks merged by plain stores):
  *   vox_scene_bricks   bricks of one scene's volume (its width a multiple of
  *                      32), 0 when it cannot take bricks; host-only
  *   vox_workspace_size_batched_volume  the batched workspace followed by the

@@ -155,11 +155,11 @@ vox_status check_generate_args(const vox_segment *segs, int64_t n, vox_dims dims
 
 // ---- the volume by brick ownership ------------------------------------------
 
-// The brick geometry of a single volume (brick_geom, with counter replicas).
+// The brick geometry of a single volume.
 bool make_geom(vox_dims dims, BrickGeom *G)
 {
     if (check_dims(dims) != VOX_OK) return false;
-    return brick_geom(dims.w, dims.h, dims.d, G, true);
+    return brick_geom(dims.w, dims.h, dims.d, G);
 }
 
 // Tensor map of the volume as a 3-D array of 32-bit words (row_words x h x d)
@@ -260,17 +260,27 @@ int grid_ctas(const void *kernel, int threads, size_t smem);
 
 // The binning passes: persistent grids (SMs x CTAs per SM, no more CTAs than
 // the segments fill), warps taking batches of segments.
+template <bool kEuclid, bool kBatched, int kPer>
+vox_status launch_bin_p(const BinParams &bp, bool scatter, int64_t n, cudaStream_t stream)
+{
+    const void *k = scatter ? reinterpret_cast<const void *>(k_bin_scatter<kEuclid, kBatched, kPer>)
+                            : reinterpret_cast<const void *>(k_bin_count<kEuclid, kBatched, kPer>);
+    int grid = grid_ctas(k, kBinThreads, 0);
+    if (grid <= 0) return VOX_ERR_CUDA;
+    constexpr int kCta = kBinWarps * 32 * kPer;  // segments of a CTA's first batches
+    grid = static_cast<int>(std::min<int64_t>(grid, (n + kCta - 1) / kCta));
+    if (scatter) k_bin_scatter<kEuclid, kBatched, kPer><<<static_cast<unsigned>(grid), kBinThreads, 0, stream>>>(bp);
+    else k_bin_count<kEuclid, kBatched, kPer><<<static_cast<unsigned>(grid), kBinThreads, 0, stream>>>(bp);
+    return cudaGetLastError() == cudaSuccess ? VOX_OK : VOX_ERR_CUDA;
+}
+
+// Segments per lane and batch: four when that leaves every warp of the grid about a
+// batch (4,864 warps), else two (the figures at bin_loop).
 template <bool kEuclid, bool kBatched>
 vox_status launch_bin_t(const BinParams &bp, bool scatter, int64_t n, cudaStream_t stream)
 {
-    const void *k = scatter ? reinterpret_cast<const void *>(k_bin_scatter<kEuclid, kBatched>)
-                            : reinterpret_cast<const void *>(k_bin_count<kEuclid, kBatched>);
-    int grid = grid_ctas(k, kBinThreads, 0);
-    if (grid <= 0) return VOX_ERR_CUDA;
-    grid = static_cast<int>(std::min<int64_t>(grid, (n + kBinWarps * kBinBatch - 1) / (kBinWarps * kBinBatch)));
-    if (scatter) k_bin_scatter<kEuclid, kBatched><<<static_cast<unsigned>(grid), kBinThreads, 0, stream>>>(bp);
-    else k_bin_count<kEuclid, kBatched><<<static_cast<unsigned>(grid), kBinThreads, 0, stream>>>(bp);
-    return cudaGetLastError() == cudaSuccess ? VOX_OK : VOX_ERR_CUDA;
+    return n >= (int64_t(1) << 18) ? launch_bin_p<kEuclid, kBatched, 4>(bp, scatter, n, stream)
+                                   : launch_bin_p<kEuclid, kBatched, 2>(bp, scatter, n, stream);
 }
 
 vox_status launch_bin(const BinParams &bp, bool euclid, bool batched, bool scatter, int64_t n, cudaStream_t stream)
@@ -597,12 +607,21 @@ BatchLayout batch_layout(int64_t n_total, int32_t n_scenes)
     return B;
 }
 
+// The scene map: several CTAs per scene while the scenes are few.
+void launch_scene_map(const SceneDesc *scenes, int32_t n_scenes, int64_t n_total, int32_t *scene_of, int32_t *status,
+                      bool list32, cudaStream_t stream)
+{
+    const int32_t parts = n_scenes <= 1024 ? 16 : 1;
+    const unsigned grid = static_cast<unsigned>(n_scenes) * static_cast<unsigned>(parts);
+    k_scene_map<<<grid, 256, 0, stream>>>(scenes, n_scenes, n_total, scene_of, status, list32 ? 1 : 0, parts);
+}
+
 // Batched volumes by bricks: the batched layout, then every scene's brick
 // numbering, then the brick arrays over all scenes' slots and the pieces.
 struct BatchBrickLayout {
     size_t sb;           // SceneBricks [n_scenes]
     size_t brick_scene;  // int32 [total_bricks]
-    VolLayout VL;        // slots = total_bricks * kPieceClasses
+    VolLayout VL;        // slots = total_bricks * kPieceClasses * replicas
     BrickGeom tot;  // n_bricks and n_slots of the whole batch (the rest unused)
 };
 
@@ -611,8 +630,8 @@ BatchBrickLayout batch_brick_layout(int64_t n_total, int32_t n_scenes, int64_t t
     BatchBrickLayout L;
     std::memset(&L.tot, 0, sizeof(L.tot));
     L.tot.n_bricks = total_bricks;
-    L.tot.n_slots = total_bricks * kPieceClasses;
-    L.tot.reps = 1;
+    L.tot.reps = counter_replicas(total_bricks);
+    L.tot.n_slots = total_bricks * kPieceClasses * L.tot.reps;
     L.sb = batch_layout(n_total, n_scenes).total;
     L.brick_scene = L.sb + align_up(sizeof(SceneBricks) * static_cast<size_t>(n_scenes));
     L.VL = vol_layout(n_total, L.tot, capacity, L.brick_scene + align_up(4 * static_cast<size_t>(total_bricks)));
@@ -1092,8 +1111,7 @@ vox_status vox_generate_batched_ex(const vox_segment *d_segs, int64_t n_total, c
     const SceneDesc *scenes = reinterpret_cast<const SceneDesc *>(d_scenes);
     int32_t *scene_of = reinterpret_cast<int32_t *>(base + B.scene_of);
     if (cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess) return VOX_ERR_CUDA;
-    k_scene_map<<<static_cast<unsigned>(n_scenes), 256, 0, s>>>(scenes, n_scenes, n_total, scene_of, d_status,
-                                                                 l32 ? 1 : 0);
+    launch_scene_map(scenes, n_scenes, n_total, scene_of, d_status, l32, s);
     if (cudaGetLastError() != cudaSuccess) return VOX_ERR_CUDA;
     if (bm && (flags & VOX_OUT_FRESH) && !bricks) {  // every scene's volume cleared (a valid table only)
         k_scene_clear<<<dim3(kSceneClearCtas, static_cast<unsigned>(n_scenes)), 256, 0, s>>>(scenes, d_status);
@@ -1142,7 +1160,7 @@ vox_status vox_generate_batched(const vox_segment *d_segs, int64_t n_total, cons
 int64_t vox_scene_bricks(vox_dims dims)
 {
     BrickGeom G;
-    if (check_dims(dims) != VOX_OK || !brick_geom(dims.w, dims.h, dims.d, &G, false)) return 0;
+    if (check_dims(dims) != VOX_OK || !brick_geom(dims.w, dims.h, dims.d, &G)) return 0;
     return G.n_bricks;
 }
 
@@ -1172,7 +1190,7 @@ vox_status vox_plan_batched(const vox_segment *d_segs, int64_t n_total, const vo
     const SceneDesc *scenes = reinterpret_cast<const SceneDesc *>(d_scenes);
     int32_t *scene_of = reinterpret_cast<int32_t *>(base + B.scene_of);
     if (cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess) return VOX_ERR_CUDA;
-    k_scene_map<<<static_cast<unsigned>(n_scenes), 256, 0, s>>>(scenes, n_scenes, n_total, scene_of, d_status, 0);
+    launch_scene_map(scenes, n_scenes, n_total, scene_of, d_status, false, s);
     if (cudaGetLastError() != cudaSuccess) return VOX_ERR_CUDA;
     int64_t V = 0, pieces = 0;
     int32_t st = 0;

@@ -54,12 +54,21 @@ struct BrickGeom {
     // pieces of similar length. Each (brick, class) has `reps` counters (segment
     // s uses replica s % reps) so that atomics on one brick spread over several
     // addresses when there are few bricks with many pieces each.
-    int32_t reps;       // 1 or 8 (segment s uses replica s & (reps - 1))
+    int32_t reps;       // 1, 8 or 32 (segment s uses replica s & (reps - 1))
     int64_t n_slots;    // n_bricks * kPieceClasses * reps
 };
 
 constexpr int kPieceClasses = 22;  // half octaves of the piece length (<= 1024)
 constexpr int64_t kMaxBricks = int64_t(1) << 26;
+
+// Counter replicas per (brick, class): a brick's counters are updated once per piece in
+// it, and updates of one address go one after another, so few bricks get more of them.
+// Binning of 48 scenes (1.17 M segments, 1,623 bricks in all), one counter per (brick,
+// class): 128 + 110 us (scatter, count), eight: 104 + 62 us.
+__host__ __device__ inline int32_t counter_replicas(int64_t bricks)
+{
+    return bricks <= 512 ? 32 : (bricks <= 32768 ? 8 : 1);
+}
 
 // Brick shape for a volume whose rows are whole 32-bit words (w % 32 == 0):
 // B0 = the largest 32 * 2^k not above min(w, 256) voxels along x (whole words),
@@ -69,9 +78,9 @@ constexpr int64_t kMaxBricks = int64_t(1) << 26;
 // and large the brick is (fewer pieces), and the brick's store writes one
 // request per brick row, so rows of 32 bytes (B0 = 256) store about three times
 // faster than rows of 16 bytes (measured: 18 against 56 us per 128 MiB volume).
-// replicas: 8 counter replicas per (brick, class) when there are few bricks
-// (a single scene), else 1 (and always 1 inside a batch of scenes).
-__host__ __device__ inline bool brick_geom(int32_t w, int32_t h, int32_t d, BrickGeom *G, bool replicas)
+// all_bricks: bricks of the whole batch that the volume belongs to (0: the volume
+// alone), which set the counter replicas.
+__host__ __device__ inline bool brick_geom(int32_t w, int32_t h, int32_t d, BrickGeom *G, int64_t all_bricks = 0)
 {
     if (w < 1 || h < 1 || d < 1 || w % 32 != 0) return false;
     int32_t b0 = 32;
@@ -102,12 +111,12 @@ __host__ __device__ inline bool brick_geom(int32_t w, int32_t h, int32_t d, Bric
         nb *= G->nb[a];
     }
     G->n_bricks = nb;
-    G->reps = (replicas && nb <= 32768) ? 8 : 1;
+    G->reps = counter_replicas(all_bricks > 0 ? all_bricks : nb);
     G->n_slots = nb * kPieceClasses * G->reps;
     return nb <= kMaxBricks && G->words <= kBrickWordsMax;
 }
 
-// A scene of a batch as the brick path sees it: its geometry (one replica), its
+// A scene of a batch as the brick path sees it: its geometry, its
 // first brick and first slot in the batch's numbering, and its volume.
 struct SceneBricks {
     BrickGeom G;
@@ -125,7 +134,7 @@ __device__ __forceinline__ int32_t piece_class_desc(int32_t len)
     return kPieceClasses - 1 - cls;
 }
 
-// Slots fit 31 bits: with 8 replicas there are at most 32768 bricks, else at
+// Slots fit 31 bits: with replicas there are at most 32768 bricks, else at
 // most 2^26 bricks and one replica.
 __device__ __forceinline__ uint32_t piece_slot(const BrickGeom &G, int32_t brick, int32_t len, int32_t rep)
 {
@@ -148,78 +157,89 @@ struct AxisCrossings {
     int32_t qs, rs;
     int32_t twoA;
 
-    __device__ __forceinline__ void init(int32_t S, int32_t E, int32_t A, int32_t N, int32_t logB)
+    // From a voxel whose coordinate on the axis is v on (the step at hand is not needed).
+    __device__ __forceinline__ void init(int32_t S, int32_t E, int32_t v, int32_t A, int32_t N, int32_t logB)
     {
-        const int32_t b0 = S >> logB, be = E >> logB;  // coordinates are inside the volume (>= 0)
+        const int32_t b0 = v >> logB, be = E >> logB;  // coordinates are inside the volume (>= 0)
         left = abs(be - b0);
         nk = kNoStep;
+        rem = qs = rs = twoA = 0;
         if (left == 0) return;
         const int32_t B = 1 << logB;
         const int32_t Q = be > b0 ? (b0 + 1) * B - S : S - b0 * B + 1;
+        // quotients below 2^22: nk <= N, and qs < 2N (there are two crossings B apart, A > B)
         twoA = 2 * A;
-        if (N <= 46340) {  // T < 2 N^2 + 2N < 2^32
-            const uint32_t T = static_cast<uint32_t>(N) * static_cast<uint32_t>(2 * Q - 1) + static_cast<uint32_t>(twoA - 1);
-            const uint32_t k = T / static_cast<uint32_t>(twoA);
-            nk = static_cast<int32_t>(k);
-            rem = static_cast<int32_t>(T - k * static_cast<uint32_t>(twoA));
-        } else {
-            const uint64_t T = static_cast<uint64_t>(N) * static_cast<uint64_t>(2 * Q - 1) + static_cast<uint64_t>(twoA - 1);
-            const uint64_t k = T / static_cast<uint64_t>(twoA);
-            nk = static_cast<int32_t>(k);
-            rem = static_cast<int32_t>(T - k * static_cast<uint64_t>(twoA));
-        }
-        if (left > 1) {  // 2NB < 2^31 (N < 2^21, B <= 256)
-            const uint32_t step = 2u * static_cast<uint32_t>(N) * static_cast<uint32_t>(B);
-            const uint32_t q = step / static_cast<uint32_t>(twoA);
-            qs = static_cast<int32_t>(q);
-            rs = static_cast<int32_t>(step - q * static_cast<uint32_t>(twoA));
-        }
+        const float rcp = __frcp_rn(static_cast<float>(twoA));
+        divmod_est(static_cast<uint64_t>(N) * static_cast<uint64_t>(2 * Q - 1) + static_cast<uint64_t>(twoA - 1), twoA,
+                   rcp, nk, rem);
+        if (left > 1) divmod_est(2ull * static_cast<uint64_t>(N) * static_cast<uint64_t>(B), twoA, rcp, qs, rs);
     }
 
-    __device__ __forceinline__ void advance()
+    // To the crossing after the one at nk, where `hit`; without a branch, since the lanes
+    // of a warp cross different axes at each of their runs.
+    __device__ __forceinline__ void advance(bool hit)
     {
-        if (--left == 0) {
-            nk = kNoStep;
-            return;
-        }
-        nk += qs;
-        rem += rs;
-        if (rem >= twoA) {
-            rem -= twoA;
-            ++nk;
-        }
+        int32_t r = rem + rs, n = nk + qs;
+        const bool over = r >= twoA;
+        r -= over ? twoA : 0;
+        n += over ? 1 : 0;
+        left -= hit ? 1 : 0;
+        nk = hit ? (left > 0 ? n : kNoStep) : nk;
+        rem = hit ? r : rem;
     }
 };
 
 // The maximal runs of consecutive steps of one segment that stay in one brick,
-// in increasing k: init() at the segment's start, then next() gives one run per
+// in increasing k: init() at a step, then next() gives one run per
 // call. Endpoints must be inside the volume. Brick indices fit 32 bits (at most
-// 2^26 bricks). kEuclid: the steps are the samples of the Euclidean-N variant,
-// N = int(|E - S|) (the crossing formula holds for any N >= max |d_a|).
-template <bool kEuclid = false>
+// 2^26 bricks). The crossing formula holds for any number of steps N >= max |d_a| (the
+// samples of the Euclidean-N variant too).
 struct PieceWalker {
     AxisCrossings ax[3];
     int32_t bstep[3];
     int32_t brick, k, N;
 
-    __device__ __forceinline__ void init(const int32_t *rec, const BrickGeom &G)
+    // At the first run that starts at step k0 or later; false when there is none (a
+    // segment's first run starts at step 0).
+    __device__ __forceinline__ bool init(const int32_t *rec, const BrickGeom &G, int32_t steps, int32_t k0)
     {
-        int32_t A[3];
-        N = 0;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            A[a] = abs(rec[3 + a] - rec[a]);
-            N = max(N, A[a]);
-        }
-        if constexpr (kEuclid) N = euclid_steps(rec);
-        brick = (rec[0] >> G.logB[0]) + G.nb[0] * ((rec[1] >> G.logB[1]) + G.nb[1] * (rec[2] >> G.logB[2]));
+        N = steps;
+        const float rcp2N = k0 > 1 ? __frcp_rn(static_cast<float>(2 * N)) : 0.0f;
         const int32_t stride[3] = {1, G.nb[0], G.nb[0] * G.nb[1]};
+        brick = 0;
+        int32_t kn = N + 1;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            ax[a].init(rec[a], rec[3 + a], A[a], N, G.logB[a]);
-            bstep[a] = rec[3 + a] >= rec[a] ? stride[a] : -stride[a];
+            const int32_t A = abs(rec[3 + a] - rec[a]);
+            const bool up = rec[3 + a] >= rec[a];
+            int32_t v = rec[a];  // the coordinate at step k0 - 1 (at step 0 when k0 is 0 or 1)
+            if (k0 > 1) {
+                int32_t q, r;
+                axis_entry(A, N, k0 - 1, rcp2N, q, r);
+                v = up ? v + q : v - q;
+            }
+            brick += (v >> G.logB[a]) * stride[a];
+            bstep[a] = up ? stride[a] : -stride[a];
+            ax[a].init(rec[a], rec[3 + a], v, A, N, G.logB[a]);
+            kn = min(kn, ax[a].nk);
         }
         k = 0;
+        if (k0 == 0) return true;
+        if (kn > N) return false;
+        enter(kn);
+        return true;
+    }
+
+    // The run that starts at step kn, where some axis enters its next brick.
+    __device__ __forceinline__ void enter(int32_t kn)
+    {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const bool hit = ax[a].nk == kn;
+            brick += hit ? bstep[a] : 0;
+            ax[a].advance(hit);
+        }
+        k = kn;
     }
 
     // The current run (brick b, first step k_lo, len steps); advances to the
@@ -231,32 +251,10 @@ struct PieceWalker {
         k_lo = k;
         len = kn - k;
         if (kn > N) return false;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (ax[a].nk == kn) {
-                brick += bstep[a];
-                ax[a].advance();
-            }
-        }
-        k = kn;
+        enter(kn);
         return true;
     }
 };
-
-// Calls f(brick, k_lo, len) for every maximal run of consecutive steps of the
-// segment that stays in one brick, in increasing k (PieceWalker in a loop).
-template <bool kEuclid = false, typename F>
-__device__ __forceinline__ void for_each_piece(const int32_t *rec, const BrickGeom &G, F &&f)
-{
-    PieceWalker<kEuclid> pw;
-    pw.init(rec, G);
-    bool more = true;
-    while (more) {
-        int32_t b, k_lo, len;
-        more = pw.next(b, k_lo, len);
-        f(b, k_lo, len);
-    }
-}
 
 // Pieces are at most kPieceMaxLen steps long: a longer run in one brick is cut
 // into parts of kPieceMaxLen (the last one shorter), so that no lane of the
@@ -317,106 +315,170 @@ __device__ __forceinline__ void load_record(const int32_t *segs, int64_t s, int3
 }
 
 // Binning work loop, shared by the counting and the scattering pass (CTAs of
-// kBinThreads threads, persistent grid). Each warp takes batches of kBinBatch
-// consecutive segments, orders each batch by length octave, longest first (a
-// counting sort in the warp's shared memory), and walks the segments in that
-// order, lane l taking the l-th of every 32: the lanes of a warp then walk
-// segments of similar length, so that a warp does not wait for one long
-// segment while its other lanes idle (lengths may span three orders of
-// magnitude). emit(slot, seg, k_lo, len) is called for every piece (runs in one
-// brick cut to at most kPieceMaxLen steps) with its slot in the batch's slot
-// numbering. A segment with an endpoint outside its volume has no pieces (the
-// count kernel reports it).
+// kBinThreads threads, persistent grid). A warp takes batches of 32 kPer consecutive
+// segments and cuts their steps into units of kBinUnit, the last one of a segment
+// shorter; a lane walks a unit: the runs (maximal runs of steps in one brick) that start
+// in it, entering the segment there by one division per axis. The whole units first,
+// 32 a round, dealt out over the lanes whichever segment they belong to, then every
+// segment's last unit, ordered by length octave: the lanes of a round walk about as many
+// runs each, whatever the mix of lengths (log-uniform lengths span three orders of
+// magnitude). emit(slot, seg, k_lo, len) is called for every piece (runs cut to at most
+// kPieceMaxLen steps) with its slot in the batch's slot numbering. A segment with an
+// endpoint outside its volume has no pieces (the count kernel reports it).
+// Bound by the L2's atomics where segments are long (counting 57 M pieces: 1.4e11
+// updates/s), else by the walk's instructions. Counting + scattering pass, us, against
+// a lane per segment in batches of 128 sorted by octave, with a branch per axis at
+// every run's end and four reservations in flight:
+//   4M log-uniform segments, 4096^3 (57 M pieces)   461 + 1295 -> 415 + 1075
+//   1M log-uniform segments, 2048^3                  73 +  222 ->  79 +  162
+//   48 uneven scenes (1.17 M segments)              132 +  196 ->  60 +  112
+//   200,000 uniform segments, 512^3                  35 +   50 ->  22 +   30
+//   1,000 uniform segments, 512 x 300 x 200          13 +   33 ->   7 +   13
+// kPer segments per lane and batch: more of them fill the rounds of equal octaves
+// better (4M: 444 + 1072 with 2, 653 + 1191 with 1), fewer keep more warps busy (the
+// 200,000: 26 + 38 with 4); launch_bin_t draws the line at 2^18 segments.
+// A lane per piece, its step and brick found by fixed-point slopes, takes about 300
+// instructions a piece (779 + 1128 us on the first).
 constexpr int kBinThreads = 256;
 constexpr int kBinWarps = kBinThreads / 32;
-constexpr int kBinPer = 4;                 // segments per lane and batch
-constexpr int kBinBatch = 32 * kBinPer;    // segments per warp batch
-constexpr int kBinOctaves = 22;            // octaves of N + 1 <= 2^21
+constexpr int kBinCtas = 4;                // CTAs per SM
+constexpr int kBinUnit = 512;              // steps
+constexpr int kBinOctaves = 10;            // of a last unit's steps, 1 .. kBinUnit
 
-template <bool kEuclid, bool kBatched, typename Emit>
+template <int kPer>
+struct BinWarpSmem {
+    static constexpr int kBatch = 32 * kPer;
+    int32_t rec[6][kBatch];   // the batch's segments
+    int32_t N[kBatch];
+    uint8_t last[kBatch];     // segments by the octave of their last unit, longest first
+    uint8_t longs[kBatch];    // segments with whole units
+    int32_t hist[32];
+};
+
+// One lane's unit: the runs of segment j (in the batch) that start at steps
+// k0 .. k0 + kBinUnit - 1.
+template <bool kBatched, int kPer, typename Emit>
+__device__ __forceinline__ void bin_unit(const BinParams &p, const BinWarpSmem<kPer> &sm, int64_t b0, int j, int32_t k0,
+                                         Emit &emit)
+{
+    const int64_t s = b0 + j;
+    int64_t slot_base;
+    const BrickGeom *Gp = segment_geom<kBatched>(p, s, slot_base);
+    const int32_t rep = static_cast<int32_t>(s) & (Gp->reps - 1);
+    int32_t r[6];
+#pragma unroll
+    for (int a = 0; a < 6; ++a) r[a] = sm.rec[a][j];
+    PieceWalker pw;
+    bool more = pw.init(r, *Gp, sm.N[j], k0);
+    int32_t b = 0, k_lo = 0, len = 0;
+    while (true) {  // a piece per iteration
+        if (len == 0) {
+            if (!more || pw.k >= k0 + kBinUnit) break;
+            more = pw.next(b, k_lo, len);
+        }
+        const int32_t part = min(len, kPieceMaxLen);
+        emit(slot_base + piece_slot(*Gp, b, part, rep), s, k_lo, part);
+        k_lo += part;
+        len -= part;
+    }
+}
+
+template <bool kEuclid, bool kBatched, int kPer, typename Emit>
 __device__ __forceinline__ void bin_loop(const BinParams &p, Emit &&emit)
 {
-    __shared__ int32_t s_recs[kBinWarps][kBinBatch * 6];
-    __shared__ uint8_t s_order[kBinWarps][kBinBatch];
-    __shared__ int32_t s_hist[kBinWarps][32];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    constexpr int kBatch = 32 * kPer;
+    __shared__ BinWarpSmem<kPer> s_bin[kBinWarps];
+    const int lane = threadIdx.x & 31;
+    BinWarpSmem<kPer> &sm = s_bin[threadIdx.x >> 5];
     const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    int32_t *const recs = s_recs[wib];
-    for (int64_t b0 = gw * kBinBatch; b0 < p.n; b0 += nw * kBinBatch) {
-        s_hist[wib][lane] = 0;
+    const uint32_t lt_mask = (1u << lane) - 1u, le_mask = lt_mask | (1u << lane);
+    for (int64_t b0 = gw * kBatch; b0 < p.n; b0 += nw * kBatch) {
+        sm.hist[lane] = 0;
         __syncwarp();
-        // the batch's records, and each segment's rank within its octave (longest first)
-        int32_t oct[kBinPer], rank[kBinPer];
+        // ---- the batch's segments; those with whole units; each one's rank in the
+        // octave of its last unit
+        int32_t oct[kPer], rank[kPer];
+        int32_t n_long = 0;
 #pragma unroll
-        for (int i = 0; i < kBinPer; ++i) {
+        for (int i = 0; i < kPer; ++i) {
             const int j = i * 32 + lane;
-            const int64_t s = b0 + j;
             oct[i] = -1;
-            if (s < p.n) {
+            rank[i] = 0;
+            bool is_long = false;
+            if (b0 + j < p.n) {
                 int32_t r[6];
-                load_record(p.segs, s, r);
+                load_record(p.segs, b0 + j, r);
+                int64_t slot_base;
+                const BrickGeom *G = segment_geom<kBatched>(p, b0 + j, slot_base);
+                if (G != nullptr && endpoints_inside(r, *G)) {
+                    int32_t N = max(abs(r[3] - r[0]), max(abs(r[4] - r[1]), abs(r[5] - r[2])));
+                    if constexpr (kEuclid) N = euclid_steps(r);
 #pragma unroll
-                for (int c = 0; c < 6; ++c) recs[6 * j + c] = r[c];
-                // the octave of N + 1 from unsigned differences: a segment with an
-                // endpoint outside the volume (skipped below) still gets a valid one
-                const uint32_t dx = static_cast<uint32_t>(abs(r[3] - r[0]));
-                const uint32_t dy = static_cast<uint32_t>(abs(r[4] - r[1]));
-                const uint32_t dz = static_cast<uint32_t>(abs(r[5] - r[2]));
-                const uint32_t octave = 31 - __clz(max(dx, max(dy, dz)) | 1u);
-                oct[i] = kBinOctaves - 1 - static_cast<int32_t>(min(octave, static_cast<uint32_t>(kBinOctaves - 1)));
-                rank[i] = atomicAdd(&s_hist[wib][oct[i]], 1);
+                    for (int a = 0; a < 6; ++a) sm.rec[a][j] = r[a];
+                    sm.N[j] = N;
+                    is_long = N >= kBinUnit;
+                    oct[i] = kBinOctaves - 1 - (31 - __clz(N % kBinUnit + 1));
+                    rank[i] = atomicAdd(&sm.hist[oct[i]], 1);
+                }
             }
+            const uint32_t m = __ballot_sync(0xffffffffu, is_long);
+            if (is_long) sm.longs[n_long + __popc(m & lt_mask)] = static_cast<uint8_t>(j);
+            n_long += __popc(m);
         }
         __syncwarp();
         // octave starts: exclusive scan of the octave counts (one per lane)
-        const int32_t h = s_hist[wib][lane];
+        const int32_t h = sm.hist[lane];
         int32_t inc = h;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
             if (lane >= o) inc += y;
         }
-        const int32_t total = __shfl_sync(0xffffffffu, inc, 31);
+        const int32_t n_valid = __shfl_sync(0xffffffffu, inc, 31);
 #pragma unroll
-        for (int i = 0; i < kBinPer; ++i) {
+        for (int i = 0; i < kPer; ++i) {
             const int32_t start = __shfl_sync(0xffffffffu, inc - h, max(oct[i], 0));
-            if (oct[i] >= 0) s_order[wib][start + rank[i]] = static_cast<uint8_t>(i * 32 + lane);
+            if (oct[i] >= 0) sm.last[start + rank[i]] = static_cast<uint8_t>(i * 32 + lane);
         }
         __syncwarp();
+        // ---- whole units: 32 long segments at a time, 32 units a round
 #pragma unroll 1
-        for (int i = 0; i < kBinPer; ++i) {
-            const int q = i * 32 + lane;
-            if (q >= total) continue;
-            const int j = s_order[wib][q];
-            const int64_t s = b0 + j;
-            int64_t slot_base;
-            const BrickGeom *Gp = segment_geom<kBatched>(p, s, slot_base);
-            if (Gp == nullptr) continue;
-            const int32_t *r = recs + 6 * j;
-            if (!endpoints_inside(r, *Gp)) continue;
-            const int32_t rep = static_cast<int32_t>(s) & (Gp->reps - 1);
-            PieceWalker<kEuclid> pw;
-            pw.init(r, *Gp);
-            bool more = true;
-            while (more) {
-                int32_t b, k_lo, len;
-                more = pw.next(b, k_lo, len);
-                while (len > 0) {
-                    const int32_t part = min(len, kPieceMaxLen);
-                    emit(slot_base + piece_slot(*Gp, b, part, rep), s, k_lo, part);
-                    k_lo += part;
-                    len -= part;
-                }
+        for (int32_t l0 = 0; l0 < n_long; l0 += 32) {
+            const int32_t own = l0 + lane < n_long ? sm.N[sm.longs[l0 + lane]] / kBinUnit : 0;
+            int32_t end = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t y = __shfl_up_sync(0xffffffffu, end, o);
+                if (lane >= o) end += y;
             }
+            const int32_t total = __shfl_sync(0xffffffffu, end, 31);
+            const int32_t pre = own > 0 ? end - own : 0x7fffffff;  // units of the segments before it
+#pragma unroll 1
+            for (int32_t base = 0; base < total; base += 32) {
+                // the lane's segment: the last one whose first unit is at or before its unit
+                const int32_t d = pre - base;
+                const uint32_t starts = __reduce_or_sync(0xffffffffu, (d > 0 && d < 32) ? 1u << d : 0u);
+                const int32_t c = __popc(__ballot_sync(0xffffffffu, d <= 0)) - 1 + __popc(starts & le_mask);
+                const int32_t first = __shfl_sync(0xffffffffu, pre, c);
+                if (base + lane < total)
+                    bin_unit<kBatched>(p, sm, b0, sm.longs[l0 + c], (base + lane - first) * kBinUnit, emit);
+                __syncwarp();
+            }
+        }
+        // ---- every segment's last unit
+#pragma unroll 1
+        for (int32_t q = lane; q < n_valid; q += 32) {
+            const int j = sm.last[q];
+            bin_unit<kBatched>(p, sm, b0, j, sm.N[j] & ~(kBinUnit - 1), emit);
         }
         __syncwarp();  // the warp's shared arrays are free for the next batch
     }
 }
 
 // Pieces per slot (persistent grid).
-template <bool kEuclid, bool kBatched = false>
-__global__ void __launch_bounds__(kBinThreads) k_bin_count(BinParams p)
+template <bool kEuclid, bool kBatched, int kPer>
+__global__ void __launch_bounds__(kBinThreads, kBinCtas) k_bin_count(BinParams p)
 {
     // single volume: no status check (this pass may run beside the count + scan
     // that resets the status word); it reads only the segments and the host's
@@ -425,23 +487,24 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(BinParams p)
     // a batch reads the scene map and numbering, valid only without an error
     // (decided by the whole warp: the walk's shuffles and votes need every lane)
     if (kBatched && __any_sync(0xffffffffu, ld_volatile_i32(p.status) != 0)) return;
-    bin_loop<kEuclid, kBatched>(p, [&](int64_t slot, int64_t, int32_t, int32_t) {
+    bin_loop<kEuclid, kBatched, kPer>(p, [&](int64_t slot, int64_t, int32_t, int32_t) {
         atomicAdd(p.brick_count + slot, 1);
     });
 }
 
 // Pieces written into their slots (persistent grid). p.G.n_slots: the number of
-// slots (all scenes' when batched). Slot reservations of up to four pieces are
-// in flight together before their stores, so the returning atomics' latency
-// overlaps.
-template <bool kEuclid, bool kBatched = false>
-__global__ void __launch_bounds__(kBinThreads) k_bin_scatter(BinParams p)
+// slots (all scenes' when batched). Bound by the latency of the returning atomics:
+// slot reservations of two pieces of a lane are in flight together before their
+// stores (4M log-uniform segments: 1075 us; four, or one held while the walk goes on:
+// 9 to 10 % more).
+template <bool kEuclid, bool kBatched, int kPer>
+__global__ void __launch_bounds__(kBinThreads, kBinCtas) k_bin_scatter(BinParams p)
 {
     // an earlier error: write nothing (decided by the whole warp, whose walk takes
     // shuffles and votes; the status word may be set by a kernel on another stream)
     if (__any_sync(0xffffffffu, ld_volatile_i32(p.status) != 0)) return;
     if (__ldg(p.brick_off + p.G.n_slots) > p.capacity) return;  // the volume falls back to atomics
-    constexpr int kBatch = 4;
+    constexpr int kBatch = 2;
     int64_t bb[kBatch];
     uint64_t val[kBatch];
     int nb = 0;
@@ -455,7 +518,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_scatter(BinParams p)
             if (e < nb) p.pieces[pos[e]] = val[e];
         nb = 0;
     };
-    bin_loop<kEuclid, kBatched>(p, [&](int64_t slot, int64_t seg, int32_t k, int32_t len) {
+    bin_loop<kEuclid, kBatched, kPer>(p, [&](int64_t slot, int64_t seg, int32_t k, int32_t len) {
 #pragma unroll
         for (int e = 0; e < kBatch; ++e)
             if (e == nb) {
@@ -639,7 +702,7 @@ __device__ __forceinline__ void take_brick(const BrickParams &p, bool overflow, 
         I.geom = p.sb[k].G;
         I.bmask = p.sb[k].mask;
         lb = b - p.sb[k].brick_base;
-        first_slot = p.sb[k].slot_base + lb * kPieceClasses;
+        first_slot = p.sb[k].slot_base + lb * kPieceClasses * I.geom.reps;
         Gt = &I.geom;
     } else {
         first_slot = b * kPieceClasses * p.G.reps;

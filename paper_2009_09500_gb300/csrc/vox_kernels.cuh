@@ -595,24 +595,26 @@ __global__ void __launch_bounds__(kGenThreads, 3) k_generate(GenParams p)
 
 // Batched scenes: check the scene table (contiguous, in order, covering all n
 // segments; dims in range; 32-bit lists need edges <= 1024) and record each
-// segment's scene. One CTA per scene. Any error goes to *status and the
-// generation kernels then write nothing.
+// segment's scene. `parts` CTAs per scene (one alone took 69 us for five scenes with
+// up to 600,000 segments). Any error goes to *status and the generation kernels then write
+// nothing.
 __global__ void __launch_bounds__(256) k_scene_map(const SceneDesc *scenes, int32_t n_scenes, int64_t n_total,
-                                                   int32_t *scene_of, int32_t *status, int32_t list32)
+                                                   int32_t *scene_of, int32_t *status, int32_t list32, int32_t parts)
 {
-    const int32_t k = blockIdx.x;
+    const int32_t k = blockIdx.x / parts, part = blockIdx.x % parts;
     const SceneDesc sd = scenes[k];
     const int64_t expect = k == 0 ? 0 : scenes[k - 1].seg_begin + scenes[k - 1].n;
     const int32_t lim = 1 << 21;
     bool ok = sd.n >= 0 && sd.seg_begin == expect && sd.seg_begin + sd.n <= n_total && sd.reserved == 0 &&
               sd.w >= 1 && sd.h >= 1 && sd.d >= 1 && sd.w <= lim && sd.h <= lim && sd.d <= lim;
     if (k == n_scenes - 1) ok = ok && sd.seg_begin + sd.n == n_total;
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && part == 0) {
         if (!ok) set_status(status, 1);  // VOX_ERR_INVALID_ARG
         else if (list32 && (sd.w > 1024 || sd.h > 1024 || sd.d > 1024)) set_status(status, 3);  // PACK_WIDTH
     }
     if (!ok) return;
-    for (int64_t i = threadIdx.x; i < sd.n; i += blockDim.x) scene_of[sd.seg_begin + i] = k;
+    for (int64_t i = part * blockDim.x + threadIdx.x; i < sd.n; i += parts * blockDim.x)
+        scene_of[sd.seg_begin + i] = k;
 }
 
 // Fresh batched volumes: scene blockIdx.y's volume zeroed by kSceneClearCtas
@@ -637,7 +639,7 @@ __global__ void __launch_bounds__(256) k_scene_clear(const SceneDesc *scenes, co
     if (tail0 + tid < words) sd.mask[tail0 + tid] = 0u;
 }
 
-// The brick numbering of a batch: every scene's geometry (one counter replica),
+// The brick numbering of a batch: every scene's geometry,
 // first brick and first slot, in scene order. One CTA: each thread takes a
 // chunk of consecutive scenes, a block scan of the chunks' brick counts gives
 // the chunks' first bricks. A scene that cannot take bricks, or a total that
@@ -658,7 +660,7 @@ __global__ void __launch_bounds__(kSceneBrickThreads) k_scene_bricks(const Scene
     int64_t own = 0;
     for (int32_t k = k0; k < k1; ++k) {  // geometry of the chunk; bases below
         SceneBricks e;
-        if (!brick_geom(scenes[k].w, scenes[k].h, scenes[k].d, &e.G, false)) {
+        if (!brick_geom(scenes[k].w, scenes[k].h, scenes[k].d, &e.G, total_bricks)) {
             s_bad = 1;
             e.G.n_bricks = 0;
         }
@@ -678,12 +680,17 @@ __global__ void __launch_bounds__(kSceneBrickThreads) k_scene_bricks(const Scene
     int64_t next = s_sum[t] - own;
     for (int32_t k = k0; k < k1; ++k) {
         sb[k].brick_base = next;
-        sb[k].slot_base = next * kPieceClasses;
-        if (ok)  // the scene of every brick (sized by total_bricks)
-            for (int64_t b = 0; b < sb[k].G.n_bricks; ++b) brick_scene[next + b] = k;
+        sb[k].slot_base = next * kPieceClasses * counter_replicas(total_bricks);
         next += sb[k].G.n_bricks;
     }
     if (t == kSceneBrickThreads - 1 && !ok) set_status(status, 1);  // VOX_ERR_INVALID_ARG
+    if (!ok) return;
+    __syncthreads();  // the scenes' bases, written above by their threads, are read by others
+    // the scene of every brick (sized by total_bricks): a warp per scene
+    for (int32_t k = t / 32; k < n_scenes; k += kSceneBrickThreads / 32) {
+        const int64_t b0 = sb[k].brick_base, nb = sb[k].G.n_bricks;
+        for (int64_t b = t % 32; b < nb; b += 32) brick_scene[b0 + b] = k;
+    }
 }
 
 // First global voxel id of every scene (and V at index n_scenes).
