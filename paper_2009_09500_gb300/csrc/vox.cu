@@ -162,7 +162,7 @@ bool make_geom(vox_dims dims, BrickGeom *G)
     return brick_geom(dims.w, dims.h, dims.d, G);
 }
 
-// Tensor map of the volume as a 3-D array of 32-bit words (row_words x h x d)
+// Tensor map of the volume as a 3-D array of 64-bit words (row_words / 2 x h x d)
 // with brick-sized boxes, for the TMA reduce-OR merge. Needs 16-byte aligned
 // rows and box rows (w and B0 multiples of 128) and a 16-byte aligned volume.
 bool make_volume_tmap(const BrickGeom &G, uint32_t *mask, CUtensorMap *out, int32_t box_z = 0)
@@ -182,25 +182,27 @@ bool make_volume_tmap(const BrickGeom &G, uint32_t *mask, CUtensorMap *out, int3
             encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
         }
     }
-    const cuuint64_t dims[3] = {static_cast<cuuint64_t>(G.row_words), static_cast<cuuint64_t>(G.dim[1]),
+    const cuuint64_t dims[3] = {static_cast<cuuint64_t>(G.row_words / 2), static_cast<cuuint64_t>(G.dim[1]),
                                 static_cast<cuuint64_t>(G.dim[2])};
     const cuuint64_t strides[2] = {4ull * G.row_words, 4ull * G.row_words * static_cast<cuuint64_t>(G.dim[1])};
-    const cuuint32_t box[3] = {static_cast<cuuint32_t>(G.bxw), static_cast<cuuint32_t>(G.B[1]),
+    const cuuint32_t box[3] = {static_cast<cuuint32_t>(G.bxw / 2), static_cast<cuuint32_t>(G.B[1]),
                                static_cast<cuuint32_t>(box_z > 0 ? box_z : G.B[2])};
     const cuuint32_t estr[3] = {1, 1, 1};
     if (box[1] > 256 || box[2] > 256) return false;
-    return encode(out, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, mask, dims, strides, box, estr,
+    return encode(out, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, mask, dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 struct VolLayout {
     int64_t n_tiles;  // scan tiles over the brick counts
-    size_t hdr;       // scan ticket at +0, brick ticket at +128
+    size_t hdr;       // scan ticket at +0, number of brick parts at +64, brick ticket at +128
     size_t count;     // int32 [n_slots]
     size_t desc;      // uint64 [n_tiles]
     size_t off;       // int64 [n_slots + 4]
     size_t cursor;    // int64 [n_slots + 1]
+    size_t hot;       // HotPart [kHotParts]
+    size_t slopes;    // SegSlopes [n]
     size_t pieces;    // uint64 [capacity]
     size_t total;
 };
@@ -242,7 +244,9 @@ VolLayout vol_layout(int64_t n, const BrickGeom &G, int64_t capacity, size_t bas
     L.desc = L.count + align_up(4 * nb);
     L.off = L.desc + align_up(8 * static_cast<size_t>(L.n_tiles));
     L.cursor = L.off + align_up(8 * (nb + 4));
-    L.pieces = L.cursor + align_up(8 * (nb + 1));
+    L.hot = L.cursor + align_up(8 * (nb + 1));
+    L.slopes = L.hot + align_up(sizeof(HotPart) * kHotParts);
+    L.pieces = L.slopes + align_up(sizeof(SegSlopes) * static_cast<size_t>(n));
     L.total = L.pieces + align_up(8 * static_cast<size_t>(capacity));
     return L;
 }
@@ -346,6 +350,7 @@ vox_status launch_count_scan(const vox_segment *segs, int64_t n, vox_dims dims, 
         bp.n = n;
         bp.G = G;
         bp.brick_count = reinterpret_cast<int32_t *>(base + VL.count);
+        bp.slopes = reinterpret_cast<SegSlopes *>(base + VL.slopes);
         bp.status = status;
         if (vox_status e = launch_bin_count(bp, euclid, false, n, stream)) return e;
     }
@@ -480,11 +485,17 @@ vox_status launch_bricks(const vox_segment *segs, int64_t n, const BrickGeom &G,
     char *base = static_cast<char *>(ws);
     if (cudaMemsetAsync(base + VL.hdr, 0, kWsAlign, stream) != cudaSuccess) return VOX_ERR_CUDA;
     if (cudaMemsetAsync(base + VL.desc, 0, VL.off - VL.desc, stream) != cudaSuccess) return VOX_ERR_CUDA;
-    BinParams bp;
+    BinParams bp{};
     bp.segs = reinterpret_cast<const int32_t *>(segs);
     bp.n = n;
     bp.G = G;
     bp.brick_count = reinterpret_cast<int32_t *>(base + VL.count);
+    bp.slopes = reinterpret_cast<SegSlopes *>(base + VL.slopes);
+    bp.hot = reinterpret_cast<HotPart *>(base + VL.hot);
+    bp.n_hot = reinterpret_cast<uint32_t *>(base + VL.hdr + 64);
+    bp.mask = mask;
+    bp.fresh = (fresh || bricked) ? 1 : 0;
+    bp.bricked = bricked ? 1 : 0;
     bp.cursor = reinterpret_cast<int64_t *>(base + VL.cursor);
     bp.brick_off = reinterpret_cast<const int64_t *>(base + VL.off);
     bp.pieces = reinterpret_cast<uint64_t *>(base + VL.pieces);
@@ -513,28 +524,30 @@ vox_status launch_bricks(const vox_segment *segs, int64_t n, const BrickGeom &G,
     k_scan<false><<<static_cast<unsigned>(VL.n_tiles), kScanThreads, 0, stream>>>(sp);
     if (count_only) return cudaGetLastError() == cudaSuccess ? VOX_OK : VOX_ERR_CUDA;
     if (vox_status e = launch_bin_scatter(bp, euclid, false, n, stream)) return e;
-    BrickParams brp;
+    BrickParams brp{};
     brp.segs = bp.segs;
     brp.G = G;
     brp.brick_off = bp.brick_off;
     brp.pieces = bp.pieces;
+    brp.slopes = bp.slopes;
+    brp.hot = bp.hot;
+    brp.n_hot = bp.n_hot;
     brp.capacity = capacity;
     brp.mask = mask;
     brp.status = status;
     brp.ticket = reinterpret_cast<uint32_t *>(base + VL.hdr + 128);
     CUtensorMap tmap;
     std::memset(&tmap, 0, sizeof(tmap));
-    brp.use_tma = (!bricked && mask != nullptr && make_volume_tmap(G, mask, &tmap)) ? 1 : 0;
+    brp.use_tma = (!bricked && mask != nullptr && make_volume_tmap(G, mask, &tmap, G.B[2] / kBrickQuarters)) ? 1 : 0;
     brp.fresh = (fresh || bricked) ? 1 : 0;
     brp.bricked = bricked ? 1 : 0;
     const size_t bsmem = sizeof(BrickSmem);
-    const void *bk = euclid ? reinterpret_cast<const void *>(k_brick_volume<true>)
-                            : reinterpret_cast<const void *>(k_brick_volume<false>);
-    if (vox_status e = allow_smem(bk, bsmem)) return e;
-    const int bgrid = grid_ctas(bk, kBrickThreads, bsmem);
+    auto bk = euclid ? (G.wide ? k_brick_volume<true, false, true> : k_brick_volume<true, false, false>)
+                     : (G.wide ? k_brick_volume<false, false, true> : k_brick_volume<false, false, false>);
+    if (vox_status e = allow_smem(reinterpret_cast<const void *>(bk), bsmem)) return e;
+    const int bgrid = grid_ctas(reinterpret_cast<const void *>(bk), kBrickThreads, bsmem);
     if (bgrid <= 0) return VOX_ERR_CUDA;
-    if (euclid) k_brick_volume<true><<<static_cast<unsigned>(bgrid), kBrickThreads, bsmem, stream>>>(brp, tmap);
-    else k_brick_volume<false><<<static_cast<unsigned>(bgrid), kBrickThreads, bsmem, stream>>>(brp, tmap);
+    bk<<<static_cast<unsigned>(bgrid), kBrickThreads, bsmem, stream>>>(brp, tmap);
     if (cudaGetLastError() != cudaSuccess) return VOX_ERR_CUDA;
     if (bricked) return VOX_OK;  // no atomics fallback for the brick-major layout (pieces must fit)
     if (euclid) return VOX_OK;   // the variant's own atomics pass is the fallback (launched by the caller)
@@ -659,6 +672,11 @@ vox_status launch_batched_bricks(const vox_segment *segs, int64_t n_total, const
     bp.n = n_total;
     bp.G = BL.tot;
     bp.brick_count = reinterpret_cast<int32_t *>(base + VL.count);
+    bp.slopes = reinterpret_cast<SegSlopes *>(base + VL.slopes);
+    bp.hot = reinterpret_cast<HotPart *>(base + VL.hot);
+    bp.n_hot = reinterpret_cast<uint32_t *>(base + VL.hdr + 64);
+    bp.fresh = fresh ? 1 : 0;
+    bp.brick_scene = brick_scene;
     bp.cursor = reinterpret_cast<int64_t *>(base + VL.cursor);
     bp.brick_off = reinterpret_cast<const int64_t *>(base + VL.off);
     bp.pieces = reinterpret_cast<uint64_t *>(base + VL.pieces);
@@ -688,6 +706,9 @@ vox_status launch_batched_bricks(const vox_segment *segs, int64_t n_total, const
     brp.G = BL.tot;
     brp.brick_off = bp.brick_off;
     brp.pieces = bp.pieces;
+    brp.slopes = bp.slopes;
+    brp.hot = bp.hot;
+    brp.n_hot = bp.n_hot;
     brp.capacity = capacity;
     brp.mask = nullptr;
     brp.status = status;
@@ -701,11 +722,11 @@ vox_status launch_batched_bricks(const vox_segment *segs, int64_t n_total, const
     CUtensorMap tmap;
     std::memset(&tmap, 0, sizeof(tmap));
     const size_t bsmem = sizeof(BrickSmem);
-    const void *bk = reinterpret_cast<const void *>(k_brick_volume<false, true>);
+    const void *bk = reinterpret_cast<const void *>(k_brick_volume<false, true, false>);
     if (vox_status e = allow_smem(bk, bsmem)) return e;
     const int bgrid = grid_ctas(bk, kBrickThreads, bsmem);
     if (bgrid <= 0) return VOX_ERR_CUDA;
-    k_brick_volume<false, true><<<static_cast<unsigned>(bgrid), kBrickThreads, bsmem, stream>>>(brp, tmap);
+    k_brick_volume<false, true, false><<<static_cast<unsigned>(bgrid), kBrickThreads, bsmem, stream>>>(brp, tmap);
     if (cudaGetLastError() != cudaSuccess) return VOX_ERR_CUDA;
     const vox_dims unused{1, 1, 1};
     return launch_generate(segs, n_total, unused, nullptr, 0, nullptr, VOX_OUT_BITMASK, ws, status, stream,
@@ -1048,6 +1069,7 @@ vox_status vox_count_bins(const vox_segment *d_segs, int64_t n, vox_dims dims, v
     bp.n = n;
     bp.G = G;
     bp.brick_count = reinterpret_cast<int32_t *>(base + VL.count);
+    bp.slopes = reinterpret_cast<SegSlopes *>(base + VL.slopes);
     return launch_bin_count(bp, false, false, n, s);
 }
 

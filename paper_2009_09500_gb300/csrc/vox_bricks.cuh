@@ -33,9 +33,14 @@
 namespace vox {
 
 constexpr int kBrickThreads = 1024;  // one CTA per SM (the bitmap takes 128 KB)
+constexpr int kBrickQuarters = 4;    // z quarters of a brick: stored and cleared by 8 warps each
 constexpr int kBrickWordsMax = 32768;  // 128 KB shared bitmap per brick
 constexpr int32_t kNoStep = 0x7fffffff;
 constexpr int32_t kStPieces = 7;  // VOX_ERR_WORKSPACE: a brick-major volume needs every piece binned
+
+// Edges up to which the slopes below are exact, for N = int(|d|) as well:
+// N < sqrt(3) 37837 < 2^16.
+constexpr int32_t kSlopeDimMax = 37837;
 
 struct BrickGeom {
     int32_t B[3];       // brick extent in voxels per axis (powers of two, B[0] >= 32)
@@ -55,6 +60,7 @@ struct BrickGeom {
     // s uses replica s % reps) so that atomics on one brick spread over several
     // addresses when there are few bricks with many pieces each.
     int32_t reps;       // 1, 8 or 32 (segment s uses replica s & (reps - 1))
+    int32_t wide;       // an edge above kSlopeDimMax: no slope table
     int64_t n_slots;    // n_bricks * kPieceClasses * reps
 };
 
@@ -112,6 +118,7 @@ __host__ __device__ inline bool brick_geom(int32_t w, int32_t h, int32_t d, Bric
     }
     G->n_bricks = nb;
     G->reps = counter_replicas(all_bricks > 0 ? all_bricks : nb);
+    G->wide = (w > kSlopeDimMax || h > kSlopeDimMax || d > kSlopeDimMax) ? 1 : 0;
     G->n_slots = nb * kPieceClasses * G->reps;
     return nb <= kMaxBricks && G->words <= kBrickWordsMax;
 }
@@ -141,6 +148,55 @@ __device__ __forceinline__ uint32_t piece_slot(const BrickGeom &G, int32_t brick
     return (static_cast<uint32_t>(brick) * kPieceClasses + static_cast<uint32_t>(piece_class_desc(len))) *
                static_cast<uint32_t>(G.reps) +
            static_cast<uint32_t>(rep);
+}
+
+// A segment as the brick kernel enters it, one 32-byte sector, written once by the
+// scattering pass: its start, directions and per axis the slope S = ceil(A 2^40 / N), so
+// that a piece is entered at any step k by a multiplication per axis,
+//   q(k) = floor((2 k A + N) / (2 N)) = floor((k S + 2^39) / 2^40),
+// and walked by 32-bit fractions. The exact positions are multiples of 1 / 2N and the
+// computed ones are above by less than k 2^-40 <= 2^-24, and by 2^-32 more for each of
+// the (at most 63) steps walked from there: below 1 / 2N for N < 2^16, so every floor
+// and carry is exact. A slope of 1 (A = N) is held as 1 - 2^-40: from the fraction 1/2
+// it gives the same floors. Volumes with larger edges enter by division instead.
+// Against the segment's record and a division per minor axis (and remainders re-biased
+// at every carry), the brick kernel takes 2823 instead of 3087 us on the 4M-segment
+// batch; the table is 128 MB there and costs the scattering pass 50 us.
+struct alignas(32) SegSlopes {
+    uint32_t xy;     // start x | y << 16
+    uint32_t z;      // start z | 2^(16 + a) where axis a decreases | major axis << 19 (first with A = N)
+    uint32_t hi;     // slopes' bits 32..39, a byte per axis
+    uint32_t lo[3];  // slopes' bits 0..31
+    uint32_t pad[2];
+};
+
+__device__ __forceinline__ SegSlopes make_slopes(const int32_t *rec, int32_t N)
+{
+    SegSlopes e;
+    e.xy = static_cast<uint32_t>(rec[0]) | (static_cast<uint32_t>(rec[1]) << 16);
+    e.z = static_cast<uint32_t>(rec[2]);
+    e.hi = 0;
+    e.pad[0] = e.pad[1] = 0;
+    uint32_t major = 3;
+    const float rcp = __frcp_rn(static_cast<float>(N));
+#pragma unroll
+    for (int a = 2; a >= 0; --a) {
+        const int32_t d = rec[3 + a] - rec[a], A = abs(d);
+        if (d < 0) e.z |= 0x10000u << a;
+        uint64_t S = (uint64_t(1) << 40) - 1;
+        if (A != N) {  // two digits of 20 bits
+            int32_t q1, r1, q2, r2;
+            divmod_est(static_cast<uint64_t>(A) << 20, N, rcp, q1, r1);
+            divmod_est(static_cast<uint64_t>(r1) << 20, N, rcp, q2, r2);
+            S = (static_cast<uint64_t>(q1) << 20) + static_cast<uint32_t>(q2) + (r2 > 0 ? 1 : 0);
+        } else {
+            major = a;
+        }
+        e.lo[a] = static_cast<uint32_t>(S);
+        e.hi |= static_cast<uint32_t>(S >> 32) << (8 * a);
+    }
+    e.z |= major << 19;
+    return e;
 }
 
 // Crossing steps of one axis. The segment's offset on the axis,
@@ -275,6 +331,21 @@ __device__ __forceinline__ bool endpoints_inside(const int32_t *r, const BrickGe
            (unsigned)r[2] < (unsigned)G.dim[2] && (unsigned)r[5] < (unsigned)G.dim[2];
 }
 
+// A brick with more than hot_pieces(total) pieces is walked in parts of about that many
+// by several CTAs, whose bitmaps are OR-ed into the volume (cleared beforehand when it
+// is a fresh one): scenes in small volumes put all their pieces into a few bricks, and
+// one CTA walks a piece in about 4 ns. Brick kernel, us, whole bricks against parts:
+// 50,000 segments in 64^3 (one brick) 202 -> 18; 100,000 in 256^3 (16 bricks) 173 -> 32;
+// 48 uneven scenes 500 -> 240; 200,000 in 512^3 (128 bricks) 105 -> 87. With 1/256 of
+// all pieces as the limit there are at most 2 * 256 parts (1/128: 43 us in 256^3).
+constexpr int64_t kHotMin = 1024;
+constexpr int kHotParts = 512;
+struct HotPart {
+    int64_t brick, lo, hi;  // the pieces [lo, hi) of a brick
+};
+
+__device__ __forceinline__ int64_t hot_pieces(int64_t total) { return max(kHotMin, (total + kHotParts / 2 - 1) / (kHotParts / 2)); }
+
 struct BinParams {
     const int32_t *segs;
     int64_t n;
@@ -285,8 +356,14 @@ struct BinParams {
     uint64_t *pieces;         // [capacity]
     int64_t capacity;
     const int32_t *status;
+    SegSlopes *slopes;        // [n], written by the scattering pass
+    HotPart *hot;             // [kHotParts] and their number (zeroed before the launch)
+    uint32_t *n_hot;
+    uint32_t *mask;           // the volume, and how it is written (as in BrickParams)
+    int32_t fresh, bricked;
     const SceneBricks *sb;    // batched: each scene's geometry and numbering (else null)
     const int32_t *scene_of;  // batched: scene of every segment
+    const int32_t *brick_scene;  // batched: scene of every brick
     int32_t n_scenes;
 };
 
@@ -383,7 +460,7 @@ __device__ __forceinline__ void bin_unit(const BinParams &p, const BinWarpSmem<k
     }
 }
 
-template <bool kEuclid, bool kBatched, int kPer, typename Emit>
+template <bool kEuclid, bool kBatched, bool kSlopes, int kPer, typename Emit>
 __device__ __forceinline__ void bin_loop(const BinParams &p, Emit &&emit)
 {
     constexpr int kBatch = 32 * kPer;
@@ -417,6 +494,7 @@ __device__ __forceinline__ void bin_loop(const BinParams &p, Emit &&emit)
 #pragma unroll
                     for (int a = 0; a < 6; ++a) sm.rec[a][j] = r[a];
                     sm.N[j] = N;
+                    if (kSlopes && G->wide == 0) p.slopes[b0 + j] = make_slopes(r, N);
                     is_long = N >= kBinUnit;
                     oct[i] = kBinOctaves - 1 - (31 - __clz(N % kBinUnit + 1));
                     rank[i] = atomicAdd(&sm.hist[oct[i]], 1);
@@ -487,12 +565,82 @@ __global__ void __launch_bounds__(kBinThreads, kBinCtas) k_bin_count(BinParams p
     // a batch reads the scene map and numbering, valid only without an error
     // (decided by the whole warp: the walk's shuffles and votes need every lane)
     if (kBatched && __any_sync(0xffffffffu, ld_volatile_i32(p.status) != 0)) return;
-    bin_loop<kEuclid, kBatched, kPer>(p, [&](int64_t slot, int64_t, int32_t, int32_t) {
+    bin_loop<kEuclid, kBatched, false, kPer>(p, [&](int64_t slot, int64_t, int32_t, int32_t) {
         atomicAdd(p.brick_count + slot, 1);
     });
 }
 
-// Pieces written into their slots (persistent grid). p.G.n_slots: the number of
+// Part c of n of a brick's words in a fresh volume set to zero, by a warp.
+__device__ __forceinline__ void clear_brick(const BrickGeom &G, int64_t lb, uint32_t *mask, bool bricked, int32_t c,
+                                            int32_t n)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t rest = lb / G.nb[0];
+    const int32_t X = static_cast<int32_t>(lb - rest * G.nb[0]) * G.bxw;
+    const int32_t Y0 = static_cast<int32_t>(rest % G.nb[1]) * G.B[1], Z0 = static_cast<int32_t>(rest / G.nb[1]) * G.B[2];
+    const int32_t plane = G.words / G.B[2];  // words per z
+    const int32_t nz = bricked ? G.B[2] : min(G.B[2], G.dim[2] - Z0);
+    const int32_t q0 = plane * (nz * c / n), q1 = plane * (nz * (c + 1) / n);
+    const bool quads = bricked || ((G.bxw & 3) == 0 && (G.row_words & 3) == 0 && (reinterpret_cast<uintptr_t>(mask) & 15u) == 0);
+    const int32_t unit = quads ? 4 : 1;
+#pragma unroll 4
+    for (int32_t q = q0 + lane * unit; q < q1; q += 32 * unit) {
+        uint32_t *w = mask + lb * G.words + q;
+        if (!bricked) {
+            const int32_t row = q >> G.log_bxw, x = X + (q & (G.bxw - 1));
+            const int32_t y = Y0 + (row & (G.B[1] - 1)), z = Z0 + (row >> G.log_b1);
+            if (y >= G.dim[1] || x >= G.row_words) continue;
+            w = mask + x + static_cast<int64_t>(G.row_words) * (y + static_cast<int64_t>(G.dim[1]) * z);
+        }
+        if (quads) *reinterpret_cast<uint4 *>(w) = make_uint4(0u, 0u, 0u, 0u);
+        else *w = 0u;
+    }
+}
+
+// The bricks to be walked in parts: their parts listed, their words of a fresh volume
+// cleared, each brick by `split` warps (one clears 64 KB in 20 to 150 us). Task
+// i = (brick, c of split) goes to warp i mod (warps of the grid), a lane each.
+template <bool kBatched>
+__device__ __forceinline__ void find_hot(const BinParams &p)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
+    const int64_t limit = hot_pieces(__ldg(p.brick_off + p.G.n_slots));
+    const int64_t slots = static_cast<int64_t>(kPieceClasses) * p.G.reps;
+    const int32_t split = p.fresh && p.G.n_bricks <= 4096 ? 32 : 1;
+    const int64_t tasks = p.G.n_bricks * split;
+    for (int64_t i0 = gw; i0 < tasks; i0 += 32 * nw) {
+        const int64_t i = i0 + lane * nw, b = i / split;
+        int64_t lo = 0, hi = 0;
+        if (i < tasks) {
+            lo = __ldg(p.brick_off + b * slots);
+            hi = __ldg(p.brick_off + (b + 1) * slots);
+        }
+        uint32_t hot = __ballot_sync(0xffffffffu, hi - lo > limit);
+        if (hi - lo > limit && i % split == 0) {
+            const int32_t parts = static_cast<int32_t>((hi - lo + limit - 1) / limit);
+            const int64_t per = ((hi - lo + parts - 1) / parts + 31) & ~int64_t(31);
+            const uint32_t at = atomicAdd(p.n_hot, static_cast<uint32_t>(parts));
+            for (int32_t e = 0; e < parts; ++e)  // in bounds: see kHotParts
+                p.hot[at + e] = HotPart{b, min64(lo + e * per, hi), min64(lo + (e + 1) * per, hi)};
+        }
+        while (p.fresh && hot) {
+            const int64_t t = i0 + (__ffs(hot) - 1) * nw, hb = t / split;
+            const int32_t c = static_cast<int32_t>(t % split);
+            hot &= hot - 1;
+            if constexpr (kBatched) {
+                const int32_t k = __ldg(p.brick_scene + hb);
+                if (p.sb[k].mask != nullptr)
+                    clear_brick(p.sb[k].G, hb - p.sb[k].brick_base, p.sb[k].mask, false, c, split);
+            } else {
+                clear_brick(p.G, hb, p.mask, p.bricked != 0, c, split);
+            }
+        }
+    }
+}
+
+// Pieces written into their slots (persistent grid), and the slope table. p.G.n_slots: the number of
 // slots (all scenes' when batched). Bound by the latency of the returning atomics:
 // slot reservations of two pieces of a lane are in flight together before their
 // stores (4M log-uniform segments: 1075 us; four, or one held while the walk goes on:
@@ -504,6 +652,7 @@ __global__ void __launch_bounds__(kBinThreads, kBinCtas) k_bin_scatter(BinParams
     // shuffles and votes; the status word may be set by a kernel on another stream)
     if (__any_sync(0xffffffffu, ld_volatile_i32(p.status) != 0)) return;
     if (__ldg(p.brick_off + p.G.n_slots) > p.capacity) return;  // the volume falls back to atomics
+    find_hot<kBatched>(p);
     constexpr int kBatch = 2;
     int64_t bb[kBatch];
     uint64_t val[kBatch];
@@ -518,7 +667,7 @@ __global__ void __launch_bounds__(kBinThreads, kBinCtas) k_bin_scatter(BinParams
             if (e < nb) p.pieces[pos[e]] = val[e];
         nb = 0;
     };
-    bin_loop<kEuclid, kBatched, kPer>(p, [&](int64_t slot, int64_t seg, int32_t k, int32_t len) {
+    bin_loop<kEuclid, kBatched, true, kPer>(p, [&](int64_t slot, int64_t seg, int32_t k, int32_t len) {
 #pragma unroll
         for (int e = 0; e < kBatch; ++e)
             if (e == nb) {
@@ -532,6 +681,7 @@ __global__ void __launch_bounds__(kBinThreads, kBinCtas) k_bin_scatter(BinParams
 
 struct BrickParams {
     const int32_t *segs;
+    const SegSlopes *slopes;
     BrickGeom G;
     const int64_t *brick_off;  // [n_slots + 1]
     const uint64_t *pieces;
@@ -539,6 +689,8 @@ struct BrickParams {
     uint32_t *mask;
     int32_t *status;
     uint32_t *ticket;  // zeroed before launch
+    const HotPart *hot;      // bricks walked in parts, and the number of parts
+    const uint32_t *n_hot;
     int32_t use_tma;   // merge by one TMA tensor reduce-OR (or store) per brick (tensor map valid)
     int32_t fresh;     // write every brick (zeros included) instead of OR-ing into the volume
     int32_t bricked;   // brick-major volume: brick b is words `words` at mask + b * words (one bulk copy)
@@ -559,6 +711,16 @@ __device__ __forceinline__ void tma_reduce_or_3d(const CUtensorMap *tmap, const 
             reinterpret_cast<uint64_t>(tmap)),
         "r"(x), "r"(y), "r"(z), "r"(smem_addr(smem))
         : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
+// ... and the 1-D form, OR-ing into global memory.
+__device__ __forceinline__ void bulk_reduce_or_1d(void *gmem, const void *smem, uint32_t bytes)
+{
+    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.or.b32 [%0], [%1], %2;" ::"l"(
+                     reinterpret_cast<uint64_t>(gmem)),
+                 "r"(smem_addr(smem)), "r"(bytes)
+                 : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
@@ -671,10 +833,26 @@ __device__ __forceinline__ void merge_brick(const uint32_t *bits, const BrickGeo
     }
 }
 
+// Merge the bitmap of a part of a brick: its nonzero words OR-ed into the volume by
+// reductions (other parts' CTAs do the same).
+__device__ __forceinline__ void merge_part(const uint32_t *bits, const BrickGeom &G, int32_t X0, int32_t Y0, int32_t Z0,
+                                           uint32_t *mask)
+{
+    for (int q = threadIdx.x; q < G.words; q += kBrickThreads) {
+        const uint32_t v = bits[q];
+        const int32_t row = q >> G.log_bxw, x = X0 / 32 + (q & (G.bxw - 1));
+        const int32_t y = Y0 + (row & (G.B[1] - 1)), z = Z0 + (row >> G.log_b1);
+        if (v != 0u && y < G.dim[1] && z < G.dim[2] && x < G.row_words)
+            atomicOr(mask + x + static_cast<int64_t>(G.row_words) * (y + static_cast<int64_t>(G.dim[1]) * z), v);
+    }
+}
+
 // A brick taken from the ticket counter: its index, its pieces [lo, hi) and its
 // origin (and, in a batch, its scene's geometry and volume).
 struct BrickInfo {
-    int64_t brick;
+    int64_t brick;       // (n_bricks when there is none left)
+    int32_t part;        // a part of a brick
+    int32_t skip;        // a brick that is walked in parts
     int64_t lo, hi;
     int32_t origin[3];
     BrickGeom geom;      // batched: the brick's scene geometry
@@ -685,13 +863,18 @@ struct BrickSmem {
     alignas(128) uint32_t bits[kBrickWordsMax];  // also the TMA source tile (128-byte aligned)
     BrickInfo info[3];   // a ring: the brick in hand, the next one, and the one after (taken ahead)
     int32_t next_group;  // next group of 32 pieces of the brick to hand to a warp
+    int32_t n_hot;       // parts of bricks (the first tickets), and the pieces beyond which
+    int64_t hot_limit;   // a brick is walked in parts (both for the thread that takes tickets)
 };
 
 // Take the next brick ticket and describe the brick (one thread).
 template <bool kBatched>
-__device__ __forceinline__ void take_brick(const BrickParams &p, bool overflow, BrickInfo &I)
+__device__ __forceinline__ void take_brick(const BrickParams &p, bool overflow, BrickSmem &sm, BrickInfo &I)
 {
-    const int64_t b = atomicAdd(p.ticket, 1u);
+    const int64_t ticket = atomicAdd(p.ticket, 1u);
+    const int64_t n_hot = sm.n_hot;
+    I.part = ticket < n_hot;
+    const int64_t b = I.part ? p.hot[ticket].brick : min64(ticket - n_hot, p.G.n_bricks);
     I.brick = b;
     if (b >= p.G.n_bricks) return;
     int64_t lb = b;  // the brick's index in its volume
@@ -712,25 +895,38 @@ __device__ __forceinline__ void take_brick(const BrickParams &p, bool overflow, 
     I.origin[1] = static_cast<int32_t>(rest % Gt->nb[1]) * Gt->B[1];
     I.origin[2] = static_cast<int32_t>(rest / Gt->nb[1]) * Gt->B[2];
     const int64_t slots_per_brick = static_cast<int64_t>(kPieceClasses) * Gt->reps;
-    I.lo = overflow ? 0 : __ldg(p.brick_off + first_slot);
-    I.hi = overflow ? 0 : __ldg(p.brick_off + first_slot + slots_per_brick);
+    if (I.part) {
+        I.lo = p.hot[ticket].lo;
+        I.hi = p.hot[ticket].hi;
+        I.skip = 0;
+    } else {
+        I.lo = overflow ? 0 : __ldg(p.brick_off + first_slot);
+        I.hi = overflow ? 0 : __ldg(p.brick_off + first_slot + slots_per_brick);
+        I.skip = I.hi - I.lo > sm.hot_limit;
+    }
 }
 
-// One CTA per brick (dynamic tickets, taken two bricks ahead by the last warp
+// One CTA per brick, or part of a brick (HotPart; dynamic tickets, the parts first, taken two bricks ahead by the last warp
 // while the others walk, so that no barrier waits for a ticket). The brick's
 // pieces arrive ordered by length class, longest first (the bucket order of the
 // binning). Group w of 32 consecutive pieces goes to warp w, further groups to
 // the warps that ask a shared counter first: the lanes of a warp walk pieces of
 // similar length (at most kPieceMaxLen steps), longest groups first. A warp's
-// first group of the next brick is loaded while it walks the current brick
-// (its pieces during the walk, their segment records after it), so that, with
+// A warp's first group of the next brick is loaded while it walks the current one
+// (its pieces during the walk, their segments' slopes after it), so that, with
 // about as many groups per brick as warps, most groups start without waiting
 // for global memory. Each lane enters its piece's segment at the piece's first
-// step (one division per minor axis) and steps through the piece with the
-// carry recurrence, OR-ing bits into the brick's shared bitmap; the bitmap is
-// then merged into the volume.
-template <bool kEuclid, bool kBatched = false>
-__global__ void __launch_bounds__(kBrickThreads) k_brick_volume(BrickParams p, const __grid_constant__ CUtensorMap tmap)
+// step and steps through the piece by the carries of its fractions (SegSlopes),
+// OR-ing bits into the brick's shared bitmap; the bitmap is then merged into the
+// volume, each z quarter by a copy of its own, so that the next brick clears a
+// quarter while the others are still being read.
+// Bound by the shared memory's atomics (32 random words take 3.5 wavefronts of two
+// cycles: 4.8 voxels per cycle and SM, 1.37 ms of the 4M-segment batch's 2.72 ms), and
+// by the CTA's wait for its longest group and for its own store between bricks. The
+// walk must not spill: 24 bytes at 64 registers cost 2.89 -> 3.29 ms (59 are used).
+template <bool kEuclid, bool kBatched, bool kWide>
+__global__ void __launch_bounds__(kBrickThreads) k_brick_volume(const __grid_constant__ BrickParams p,
+                                                                const __grid_constant__ CUtensorMap tmap)
 {
     extern __shared__ __align__(128) unsigned char brick_smem_raw[];
     BrickSmem &sm = *reinterpret_cast<BrickSmem *>(brick_smem_raw);
@@ -751,16 +947,28 @@ __global__ void __launch_bounds__(kBrickThreads) k_brick_volume(BrickParams p, c
     const bool async_store = p.use_tma || p.bricked;  // the bitmap leaves by the bulk-copy unit
     const int64_t total_bricks = p.G.n_bricks;
     using St = typename std::conditional<kEuclid, EuclidStepper<uint32_t, uint32_t>, Stepper<uint32_t, uint32_t>>::type;
+    // a piece's slope table entry (in a wide volume the piece's segment is entered by division)
+    auto load_slopes = [&](uint64_t piece, uint4 &a, uint2 &b) {
+        const uint4 *e = reinterpret_cast<const uint4 *>(p.slopes + (piece & 0xffffffffull));
+        a = __ldg(e);
+        b = __ldg(reinterpret_cast<const uint2 *>(e + 1));
+    };
     // this warp's first group of the brick in hand, when loaded ahead
     bool have_pref = false;
     uint64_t pc_pref = 0;
-    int32_t rec_pref[6] = {0, 0, 0, 0, 0, 0};
+    uint4 sa_pref = make_uint4(0u, 0u, 0u, 0u);
+    uint2 sb_pref = make_uint2(0u, 0u);
+    // the quarter of the bitmap that this thread's 8 warps store and clear
+    const int quarter = t / (kBrickThreads / kBrickQuarters);
+    const bool leader = t % (kBrickThreads / kBrickQuarters) == 0;
     // ring positions of the brick in hand, the next one and the one after
     int cur = 0, nxt = 1, aft = 2;
     const bool taker = t == kBrickThreads - 32;  // lane 0 of the last warp takes the tickets
     if (taker) {
-        take_brick<kBatched>(p, overflow, sm.info[0]);
-        take_brick<kBatched>(p, overflow, sm.info[1]);
+        sm.n_hot = overflow ? 0 : static_cast<int32_t>(__ldg(p.n_hot));
+        sm.hot_limit = hot_pieces(__ldg(p.brick_off + p.G.n_slots));
+        take_brick<kBatched>(p, overflow, sm, sm.info[0]);
+        take_brick<kBatched>(p, overflow, sm, sm.info[1]);
     }
     while (true) {
         __syncthreads();
@@ -769,15 +977,18 @@ __global__ void __launch_bounds__(kBrickThreads) k_brick_volume(BrickParams p, c
         const int64_t b = I.brick;
         if (b >= total_bricks) break;
         const BrickGeom &G = kBatched ? I.geom : p.G;
+        const bool wide = kBatched ? G.wide != 0 : kWide;
         const int32_t X0 = I.origin[0], Y0 = I.origin[1], Z0 = I.origin[2];
         const uint32_t bw = static_cast<uint32_t>(G.B[0]);
         const uint32_t bwh = static_cast<uint32_t>(G.B[0]) * static_cast<uint32_t>(G.B[1]);
-        const int64_t lo = I.lo, cnt = I.hi - I.lo;
+        // below 2^31: a brick beyond the limit of hot_pieces is walked in parts
+        const uint64_t *const pieces = p.pieces + I.lo;
+        const int32_t cnt = static_cast<int32_t>(I.hi - I.lo);
         const bool next_ok = NI.brick < total_bricks;
-        const int64_t lo_n = NI.lo, cnt_n = next_ok ? NI.hi - NI.lo : 0;
-        if (cnt == 0 && !p.fresh) {
+        const int32_t cnt_n = next_ok ? static_cast<int32_t>(NI.hi - NI.lo) : 0;
+        if ((cnt == 0 && !p.fresh) || I.skip) {
             have_pref = false;
-            if (taker) take_brick<kBatched>(p, overflow, sm.info[aft]);  // read by no one now
+            if (taker) take_brick<kBatched>(p, overflow, sm, sm.info[aft]);  // read by no one now
             const int c = cur;
             cur = nxt;
             nxt = aft;
@@ -787,83 +998,138 @@ __global__ void __launch_bounds__(kBrickThreads) k_brick_volume(BrickParams p, c
         // the warp's first group (group `warp`): loaded ahead, or its pieces now
         // (their records after the clear, so that the latency overlaps it)
         int32_t grp = warp;
-        int64_t j = static_cast<int64_t>(grp) * 32 + lane;
-        uint64_t pc = have_pref ? pc_pref : (j < cnt ? __ldg(p.pieces + lo + j) : 0ull);
-        int32_t rec[6];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) rec[c] = rec_pref[c];
+        int32_t j = t;
+        uint64_t pc = have_pref ? pc_pref : (j < cnt ? __ldg(pieces + j) : 0ull);
+        uint4 sa = sa_pref;
+        uint2 sb = sb_pref;
         // the next brick's first group for this warp: its pieces now, consumed after the walk
-        const int64_t jn = static_cast<int64_t>(warp) * 32 + lane;
-        const uint64_t pc_n = jn < cnt_n ? __ldg(p.pieces + lo_n + jn) : 0ull;
-        if (t == 0) {
-            sm.next_group = kBrickThreads / 32;  // groups beyond the first round, on demand
-            if (async_store) bulk_wait_read_all();  // the previous brick's copy must have read the tile
+        const uint64_t pc_n = t < cnt_n ? __ldg(p.pieces + NI.lo + t) : 0ull;
+        if (t == 0) sm.next_group = kBrickThreads / 32;  // groups beyond the first round, on demand
+        // each quarter is cleared as soon as its own copy has been read
+        if (async_store) {
+            if (leader) bulk_wait_read_all();
+            asm volatile("bar.sync %0, %1;" ::"r"(quarter + 1), "n"(kBrickThreads / kBrickQuarters) : "memory");
         }
-        __syncthreads();
-        {  // words is a multiple of 4 (bxw * B1 * B2 with B1 * B2 >= 8)
-            uint4 *z = reinterpret_cast<uint4 *>(sm.bits);
-            for (int q = t; q < G.words / 4; q += kBrickThreads) z[q] = make_uint4(0u, 0u, 0u, 0u);
+        {  // a quarter's words are a multiple of 4
+            const int n4 = G.words / kBrickQuarters / 4;
+            uint4 *z = reinterpret_cast<uint4 *>(sm.bits) + quarter * n4;
+            for (int q = t % (kBrickThreads / kBrickQuarters); q < n4; q += kBrickThreads / kBrickQuarters)
+                z[q] = make_uint4(0u, 0u, 0u, 0u);
         }
-        if (!have_pref && j < cnt) load_record(p.segs, static_cast<int64_t>(pc & 0xffffffffull), rec);
+        if (!have_pref && j < cnt && !wide) load_slopes(pc, sa, sb);
         __syncthreads();
         // the brick after the next one: its ticket is taken while the CTA walks this
         // one (its ring slot held the brick before this one, read by no one now)
-        if (taker) take_brick<kBatched>(p, overflow, sm.info[aft]);
+        if (taker) take_brick<kBatched>(p, overflow, sm, sm.info[aft]);
         // brick-local bit index of (x, y, z): (x - X0) + B0 (y - Y0) + B0 B1 (z - Z0),
         // kept modulo 2^32 while stepping (only the local value is ever used)
         const uint32_t origin = static_cast<uint32_t>(X0) + static_cast<uint32_t>(Y0) * bw +
                                 static_cast<uint32_t>(Z0) * bwh;
+        // one shared-memory atomic per voxel: cheaper than branching to merge runs of the
+        // same word (measured on both workload shapes); repeated samples of the Euclidean
+        // variant set the same bit again
+        auto put = [&](uint32_t L) { atomicOr(sm.bits + (L >> 5), 1u << (L & 31u)); };
 #pragma unroll 1
-        while (static_cast<int64_t>(grp) * 32 < cnt) {
+        while (grp * 32 < cnt) {
             if (j < cnt) {
                 const int32_t len = static_cast<int32_t>(pc >> 54) + 1;
-                St st;
-                st.enter(rec, static_cast<int32_t>((pc >> 32) & 0x3fffffull), bw, bwh);
-                st.L -= origin;
-                // one shared-memory atomic per voxel: cheaper than branching to
-                // merge runs of the same word (measured on both workload shapes);
-                // repeated samples of the Euclidean variant set the same bit again
-                int32_t e = 0;
-                for (; e + 8 <= len; e += 8) {
-#pragma unroll
-                    for (int v = 0; v < 8; ++v) {
-                        atomicOr(sm.bits + (st.L >> 5), 1u << (st.L & 31u));
+                const int32_t k = static_cast<int32_t>((pc >> 32) & 0x3fffffull);
+                if (wide) {
+                    int32_t rec[6];
+                    load_record(p.segs, static_cast<int64_t>(pc & 0xffffffffull), rec);
+                    St st;
+                    st.enter(rec, k, bw, bwh);
+                    st.L -= origin;
+                    for (int32_t e = 0; e < len; ++e) {
+                        put(st.L);
                         st.template step<false, true>();
                     }
-                }
-                for (; e < len; ++e) {
-                    atomicOr(sm.bits + (st.L >> 5), 1u << (st.L & 31u));
-                    st.template step<false, true>();
+                } else {
+                    // the voxel at step k, its fractions and the signed strides
+                    uint32_t f[3], s[3], d[3];
+                    const uint32_t v[3] = {sa.x & 0xffffu, sa.x >> 16, sa.y & 0xffffu}, lo[3] = {sa.w, sb.x, sb.y},
+                                   st[3] = {1u, bw, bwh};
+                    uint32_t L = 0u - origin;
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        const uint32_t hi = (sa.z >> (8 * a)) & 0xffu;
+                        const uint64_t P = static_cast<uint64_t>(static_cast<uint32_t>(k)) * lo[a] + (uint64_t(1) << 39) +
+                                           (static_cast<uint64_t>(static_cast<uint32_t>(k) * hi) << 32);
+                        const bool down = (sa.y & (0x10000u << a)) != 0u;
+                        const uint32_t q = static_cast<uint32_t>(P >> 40);
+                        L += (down ? v[a] - q : v[a] + q) * st[a];
+                        d[a] = down ? 0u - st[a] : st[a];
+                        f[a] = static_cast<uint32_t>(P >> 8) + 1u;
+                        s[a] = (hi << 24) | (lo[a] >> 8);
+                        s[a] += s[a] != 0xffffffffu && (lo[a] & 0xffu) != 0u ? 1u : 0u;
+                    }
+                    if constexpr (kEuclid) {
+#pragma unroll 4
+                        for (int32_t e = 0; e < len; ++e) {
+                            put(L);
+#pragma unroll
+                            for (int a = 0; a < 3; ++a) L += add_carry(f[a], s[a]) * d[a];
+                        }
+                    } else {
+                        // the major axis moves at every step
+                        const uint32_t m = sa.y >> 19;
+                        const uint32_t dm = m == 0 ? d[0] : (m == 1 ? d[1] : d[2]);
+                        const uint32_t db = m == 0 ? d[1] : d[0], dc = m == 2 ? d[1] : d[2];
+                        uint32_t fb = m == 0 ? f[1] : f[0], fc = m == 2 ? f[1] : f[2];
+                        const uint32_t sb_ = m == 0 ? s[1] : s[0], sc = m == 2 ? s[1] : s[2];
+                        int32_t e = 0;
+                        for (; e + 8 <= len; e += 8) {
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                put(L);
+                                const uint32_t cb = add_carry(fb, sb_), cc = add_carry(fc, sc);
+                                L += dm + cb * db + cc * dc;
+                            }
+                        }
+                        for (; e < len; ++e) {
+                            put(L);
+                            const uint32_t cb = add_carry(fb, sb_), cc = add_carry(fc, sc);
+                            L += dm + cb * db + cc * dc;
+                        }
+                    }
                 }
             }
             __syncwarp();
             if (lane == 0) grp = atomicAdd(&sm.next_group, 1);
             grp = __shfl_sync(0xffffffffu, grp, 0);
-            j = static_cast<int64_t>(grp) * 32 + lane;
+            j = grp * 32 + lane;
             if (j < cnt) {
-                pc = __ldg(p.pieces + lo + j);
-                load_record(p.segs, static_cast<int64_t>(pc & 0xffffffffull), rec);
+                pc = __ldg(pieces + j);
+                if (!wide) load_slopes(pc, sa, sb);
             }
         }
-        // the next brick's first group: its pieces have arrived, now their records
+        // the next brick's first group: its pieces have arrived, now their slopes
         have_pref = next_ok;
         pc_pref = pc_n;
-        if (jn < cnt_n) load_record(p.segs, static_cast<int64_t>(pc_n & 0xffffffffull), rec_pref);
+        if (t < cnt_n && !(kBatched ? NI.geom.wide != 0 : kWide)) load_slopes(pc_n, sa_pref, sb_pref);
         __syncthreads();
-        if (p.bricked) {
-            if (t == 0) {
-                fence_proxy_async_smem();
-                bulk_store_1d(p.mask + b * G.words, sm.bits, static_cast<uint32_t>(G.words) * 4u);
-            }
-        } else if (p.use_tma) {
-            if (t == 0) {
-                fence_proxy_async_smem();  // the bitmap's generic writes, visible to the TMA unit
-                if (p.fresh) tma_store_3d(&tmap, sm.bits, X0 / 32, Y0, Z0);
-                else tma_reduce_or_3d(&tmap, sm.bits, X0 / 32, Y0, Z0);
+        if (async_store) {
+            const int32_t part = G.words / kBrickQuarters;
+            const int32_t z = Z0 + quarter * (G.B[2] / kBrickQuarters);
+            if (leader) {
+                fence_proxy_async_smem();  // the bitmap's generic writes, visible to the bulk-copy unit
+                if (p.bricked) {
+                    uint32_t *const dst = p.mask + b * G.words + quarter * part;
+                    if (I.part) bulk_reduce_or_1d(dst, sm.bits + quarter * part, static_cast<uint32_t>(part) * 4u);
+                    else bulk_store_1d(dst, sm.bits + quarter * part, static_cast<uint32_t>(part) * 4u);
+                } else if (z >= G.dim[2]) {
+                    // the quarter lies beyond the volume
+                } else if (p.fresh && !I.part)
+                    tma_store_3d(&tmap, sm.bits + quarter * part, X0 / 64, Y0, z);
+                else
+                    tma_reduce_or_3d(&tmap, sm.bits + quarter * part, X0 / 64, Y0, z);
             }
         } else {
             uint32_t *const mask = kBatched ? I.bmask : p.mask;
-            if (mask != nullptr) merge_brick(sm.bits, G, X0, Y0, Z0, mask, p.fresh != 0);
+            if (mask != nullptr) {
+                if (I.part) merge_part(sm.bits, G, X0, Y0, Z0, mask);
+                else merge_brick(sm.bits, G, X0, Y0, Z0, mask, p.fresh != 0);
+            }
             __syncthreads();
         }
         const int c = cur;
@@ -871,7 +1137,7 @@ __global__ void __launch_bounds__(kBrickThreads) k_brick_volume(BrickParams p, c
         nxt = aft;
         aft = c;
     }
-    if (async_store && t == 0) bulk_wait_all();  // copies complete before the CTA's memory goes
+    if (async_store && leader) bulk_wait_all();  // copies complete before the CTA's memory goes
 }
 
 // Brick-major volume -> row-major volume: one warp per volume row (y, z), lanes
@@ -936,7 +1202,7 @@ __global__ void __launch_bounds__(32) k_unbrick_tma(const uint32_t *bricked, Bri
             break;
         }
         phase ^= 1u;
-        tma_store_3d(&tmap, buf, X0 / 32, Y0, Z0 + h * part_rows);
+        tma_store_3d(&tmap, buf, X0 / 64, Y0, Z0 + h * part_rows);
     }
     bulk_wait_all();
 }

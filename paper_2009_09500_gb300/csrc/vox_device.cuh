@@ -18,6 +18,9 @@
 
 namespace vox {
 
+__device__ __forceinline__ int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
+__device__ __forceinline__ int64_t max64(int64_t a, int64_t b) { return a > b ? a : b; }
+
 // ------------------------------------------------------------------ PTX helpers
 __device__ __forceinline__ uint64_t globaltimer_ns()
 {

@@ -6,7 +6,7 @@ voxels and the documented brick shape, whole volumes against the oracle."""
 import numpy as np
 import pytest
 
-from gpu_util import brick_pieces_expected, get_oracle, run_gpu
+from gpu_util import brick_pieces_expected, bricked_from_row_major, get_oracle, run_gpu
 from paper_2009_09500_gb300 import batching, vox, workloads
 
 pytestmark = pytest.mark.gpu
@@ -50,3 +50,23 @@ def test_binning_batched_few_and_many_bricks():
         assert int(b.status.item()) == 0
         for m, s in zip(b.masks, scenes):
             assert np.array_equal(m.cpu().numpy().view(np.uint32), O.bitmask(s.segs, s.dims))
+
+
+@pytest.mark.parametrize("dims", [(64, 64, 64), (128, 128, 96), (160, 70, 130), (256, 256, 100)])
+@pytest.mark.parametrize("flags", [vox.OUT_BITMASK, vox.OUT_BITMASK | vox.OUT_FRESH, vox.OUT_BITMASK | vox.OUT_BRICKED])
+def test_bricks_walked_in_parts(dims, flags):
+    """Many pieces in few bricks: several CTAs walk a brick, whose bits are OR-ed into a
+    volume that is kept, cleared first, or brick-major; over stale bits."""
+    rng = np.random.default_rng(sum(dims))
+    segs = workloads.uniform_segments(rng, 9000, dims)
+    bricked = bool(flags & vox.OUT_BRICKED)
+    words = vox.vox_mask_words_bricked(dims) if bricked else vox.vox_mask_words(dims)
+    init = rng.integers(0, 2**32, size=words, dtype=np.uint64).astype(np.uint32)
+    r = run_gpu(segs, dims, flags, mask_init=init, pieces="plan", mask_words=words)
+    want = get_oracle().bitmask(segs, dims)
+    if bricked:
+        want = bricked_from_row_major(want, dims)
+    elif not flags & vox.OUT_FRESH:
+        want = want | init
+    assert r["status"] == 0
+    assert np.array_equal(r["mask"], want)
