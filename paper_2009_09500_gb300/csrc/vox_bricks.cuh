@@ -432,6 +432,25 @@ struct BinWarpSmem {
     int32_t hist[32];
 };
 
+// Volumes of at most kFewBricks bricks: the lanes of a warp mostly ask for a few slots,
+// so those that ask for the same one together share one update (and the segments of a
+// warp one replica). Scattering and counting pass, us: 50,000 segments in 64^3 14 + 8 ->
+// 9 + 4, 48 uneven scenes 117 + 59 -> 106 + 53.
+constexpr int64_t kFewBricks = 8;
+
+// The lanes active here with the same slot: the group, its leader, and the lane's rank.
+struct SlotGroup {
+    uint32_t lanes;
+    int leader, rank;
+
+    __device__ __forceinline__ explicit SlotGroup(int64_t slot)
+    {
+        lanes = __match_any_sync(__activemask(), static_cast<unsigned long long>(slot));
+        leader = __ffs(lanes) - 1;
+        rank = __popc(lanes & ((1u << (threadIdx.x & 31)) - 1u));
+    }
+};
+
 // One lane's unit: the runs of segment j (in the batch) that start at steps
 // k0 .. k0 + kBinUnit - 1.
 template <bool kBatched, int kPer, typename Emit>
@@ -441,7 +460,8 @@ __device__ __forceinline__ void bin_unit(const BinParams &p, const BinWarpSmem<k
     const int64_t s = b0 + j;
     int64_t slot_base;
     const BrickGeom *Gp = segment_geom<kBatched>(p, s, slot_base);
-    const int32_t rep = static_cast<int32_t>(s) & (Gp->reps - 1);
+    const bool few = Gp->n_bricks <= kFewBricks;
+    const int32_t rep = static_cast<int32_t>(few ? s >> 5 : s) & (Gp->reps - 1);
     int32_t r[6];
 #pragma unroll
     for (int a = 0; a < 6; ++a) r[a] = sm.rec[a][j];
@@ -454,7 +474,7 @@ __device__ __forceinline__ void bin_unit(const BinParams &p, const BinWarpSmem<k
             more = pw.next(b, k_lo, len);
         }
         const int32_t part = min(len, kPieceMaxLen);
-        emit(slot_base + piece_slot(*Gp, b, part, rep), s, k_lo, part);
+        emit(slot_base + piece_slot(*Gp, b, part, rep), s, k_lo, part, few);
         k_lo += part;
         len -= part;
     }
@@ -565,8 +585,13 @@ __global__ void __launch_bounds__(kBinThreads, kBinCtas) k_bin_count(BinParams p
     // a batch reads the scene map and numbering, valid only without an error
     // (decided by the whole warp: the walk's shuffles and votes need every lane)
     if (kBatched && __any_sync(0xffffffffu, ld_volatile_i32(p.status) != 0)) return;
-    bin_loop<kEuclid, kBatched, false, kPer>(p, [&](int64_t slot, int64_t, int32_t, int32_t) {
-        atomicAdd(p.brick_count + slot, 1);
+    bin_loop<kEuclid, kBatched, false, kPer>(p, [&](int64_t slot, int64_t, int32_t, int32_t, bool few) {
+        if (few) {
+            const SlotGroup g(slot);
+            if (g.rank == 0) atomicAdd(p.brick_count + slot, __popc(g.lanes));
+        } else {
+            atomicAdd(p.brick_count + slot, 1);
+        }
     });
 }
 
@@ -667,7 +692,17 @@ __global__ void __launch_bounds__(kBinThreads, kBinCtas) k_bin_scatter(BinParams
             if (e < nb) p.pieces[pos[e]] = val[e];
         nb = 0;
     };
-    bin_loop<kEuclid, kBatched, true, kPer>(p, [&](int64_t slot, int64_t seg, int32_t k, int32_t len) {
+    bin_loop<kEuclid, kBatched, true, kPer>(p, [&](int64_t slot, int64_t seg, int32_t k, int32_t len, bool few) {
+        if (few) {
+            const SlotGroup g(slot);
+            unsigned long long at = 0;
+            if (g.rank == 0)
+                at = atomicAdd(reinterpret_cast<unsigned long long *>(p.cursor + slot),
+                               static_cast<unsigned long long>(__popc(g.lanes)));
+            at = __shfl_sync(g.lanes, at, g.leader);
+            p.pieces[at + g.rank] = pack_piece(seg, k, len);
+            return;
+        }
 #pragma unroll
         for (int e = 0; e < kBatch; ++e)
             if (e == nb) {
