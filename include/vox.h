@@ -222,7 +222,7 @@ vox_status vox_euclid_plan(const vox_segment *d_segs, int64_t n, vox_dims dims, 
  *                           int32[6]); VOX_ERR_INVALID_ARG when w % 32 != 0
  *   vox_unbrick             device brick-major volume -> device row-major volume
  *                           (vox_mask_words(dims) words), asynchronous on stream;
- *                           half bricks through TMA when w and B0 are multiples of
+ *                           quarter bricks through TMA when w and B0 are multiples of
  *                           128 and both buffers 16-byte aligned (its bounded
  *                           waits report VOX_ERR_TIMEOUT to d_status, which may be
  *                           NULL), else one warp per volume row

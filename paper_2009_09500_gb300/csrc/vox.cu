@@ -1267,7 +1267,7 @@ vox_status vox_unbrick(const uint32_t *d_bricked, vox_dims dims, uint32_t *d_mas
     if (!aligned(d_bricked, 4) || !aligned(d_mask, 4)) return VOX_ERR_ALIGNMENT;
     const int sms = sm_count();
     if (sms <= 0) return VOX_ERR_CUDA;
-    // half bricks through the bulk-copy unit when the volume takes brick-shaped
+    // quarter bricks through the bulk-copy unit when the volume takes brick-shaped
     // TMA boxes (w and B0 multiples of 128, 16-byte aligned buffers)
     CUtensorMap tmap;
     std::memset(&tmap, 0, sizeof(tmap));
