@@ -304,16 +304,20 @@ vox_status launch_bin_scatter(const BinParams &bp, bool euclid, bool batched, in
     return launch_bin(bp, euclid, batched, true, n, stream);
 }
 
+// Whether a single scene's count + scan is one CTA's (k_scan_small), which resets the
+// status word itself: the caller does that otherwise.
+bool small_scan(int64_t n) { return n > 0 && n <= kSmallScan && g_stall_tile.load() < 0; }
+
 // Count + scan. With a brick workspace it also zeroes the brick arrays and
 // counts every segment's pieces per brick (k_bin_count).
 vox_status launch_count_scan(const vox_segment *segs, int64_t n, vox_dims dims, int32_t *counts,
                              int64_t *offsets_out, void *ws, size_t ws_bytes, int32_t *status, cudaStream_t stream,
                              const SceneDesc *scenes = nullptr, const int32_t *scene_of = nullptr,
-                             int32_t n_scenes = 0, bool euclid = false)
+                             int32_t n_scenes = 0, bool euclid = false, bool small = false)
 {
     const WsLayout L = ws_layout(n);
     char *base = static_cast<char *>(ws);
-    if (cudaMemsetAsync(base, 0, L.offsets, stream) != cudaSuccess) return VOX_ERR_CUDA;
+    if (!small && cudaMemsetAsync(base, 0, L.offsets, stream) != cudaSuccess) return VOX_ERR_CUDA;
     BrickGeom G;
     const size_t vbase = euclid ? euclid_layout(n).total : 0;
     const bool bins = scene_of == nullptr && uses_bricks(n, dims, ws_bytes, &G, vbase);
@@ -342,7 +346,9 @@ vox_status launch_count_scan(const vox_segment *segs, int64_t n, vox_dims dims, 
     p.scenes = scenes;
     p.scene_of = scene_of;
     p.n_scenes = n_scenes;
-    if (euclid) k_scan<true, true><<<static_cast<unsigned>(L.n_tiles), kScanThreads, 0, stream>>>(p);
+    if (small && euclid) k_scan_small<true><<<1, kSmallThreads, 0, stream>>>(p);
+    else if (small) k_scan_small<false><<<1, kSmallThreads, 0, stream>>>(p);
+    else if (euclid) k_scan<true, true><<<static_cast<unsigned>(L.n_tiles), kScanThreads, 0, stream>>>(p);
     else k_scan<true><<<static_cast<unsigned>(L.n_tiles), kScanThreads, 0, stream>>>(p);
     if (bins) {
         BinParams bp{};
@@ -855,14 +861,14 @@ vox_status launch_euclid_list(const EuclidParams &p, cudaStream_t stream)
 // fit) or by the run walk's atomics.
 vox_status launch_euclid(const vox_segment *segs, int64_t n, vox_dims dims, void *list, int64_t capacity,
                          uint32_t *mask, int flags, int64_t *seg_off, void *ws, size_t ws_bytes, int32_t *status,
-                         cudaStream_t stream, bool count_only)
+                         cudaStream_t stream, bool count_only, bool small)
 {
     const EuclidLayout E = euclid_layout(n);
     char *base = static_cast<char *>(ws);
     BrickGeom G;
     const bool bricks = uses_bricks(n, dims, ws_bytes, &G, E.total);
     if (vox_status e = launch_count_scan(segs, n, dims, nullptr, nullptr, ws, ws_bytes, status, stream, nullptr,
-                                         nullptr, 0, true))
+                                         nullptr, 0, true, small))
         return e;
     if (cudaMemsetAsync(base + E.hdr, 0, kWsAlign, stream) != cudaSuccess) return VOX_ERR_CUDA;
     if (cudaMemsetAsync(base + E.desc, 0, E.off - E.desc, stream) != cudaSuccess) return VOX_ERR_CUDA;
@@ -1039,7 +1045,8 @@ vox_status vox_count(const vox_segment *d_segs, int64_t n, vox_dims dims, int32_
     if (n > 0 && !aligned(d_segs, 16)) return VOX_ERR_ALIGNMENT;
     if (d_ws == nullptr || !aligned(d_ws, kWsAlign) || ws_bytes < ws_layout(n).total) return VOX_ERR_WORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess) return VOX_ERR_CUDA;
+    const bool small = small_scan(n);
+    if (!small && cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess) return VOX_ERR_CUDA;
     if (n == 0) {
         const WsLayout L = ws_layout(0);
         if (cudaMemsetAsync(static_cast<char *>(d_ws) + L.offsets, 0, 4 * sizeof(int64_t), s) != cudaSuccess)
@@ -1047,7 +1054,8 @@ vox_status vox_count(const vox_segment *d_segs, int64_t n, vox_dims dims, int32_
         if (d_offsets && cudaMemsetAsync(d_offsets, 0, sizeof(int64_t), s) != cudaSuccess) return VOX_ERR_CUDA;
         return VOX_OK;
     }
-    return launch_count_scan(d_segs, n, dims, d_counts, d_offsets, d_ws, ws_bytes, d_status, s);
+    return launch_count_scan(d_segs, n, dims, d_counts, d_offsets, d_ws, ws_bytes, d_status, s, nullptr, nullptr, 0,
+                             false, small);
 }
 
 vox_status vox_count_bins(const vox_segment *d_segs, int64_t n, vox_dims dims, void *d_ws, size_t ws_bytes,
@@ -1080,9 +1088,11 @@ vox_status vox_generate(const vox_segment *d_segs, int64_t n, vox_dims dims, voi
                                            d_status))
         return e;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess) return VOX_ERR_CUDA;
+    const bool small = small_scan(n);
+    if (!small && cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess) return VOX_ERR_CUDA;
     if (n > 0) {
-        if (vox_status e = launch_count_scan(d_segs, n, dims, nullptr, nullptr, d_ws, ws_bytes, d_status, s))
+        if (vox_status e = launch_count_scan(d_segs, n, dims, nullptr, nullptr, d_ws, ws_bytes, d_status, s, nullptr,
+                                             nullptr, 0, false, small))
             return e;
     }
     return launch_outputs(d_segs, n, dims, d_list, list_capacity, d_mask, flags, d_ws, ws_bytes, d_status, s);
@@ -1313,7 +1323,8 @@ vox_status vox_euclid_generate(const vox_segment *d_segs, int64_t n, vox_dims di
     if (n >= 0 && ws_bytes < euclid_layout(n).total) return VOX_ERR_WORKSPACE;
     if (d_offsets != nullptr && !aligned(d_offsets, 8)) return VOX_ERR_ALIGNMENT;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess) return VOX_ERR_CUDA;
+    const bool small = small_scan(n);
+    if (!small && cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess) return VOX_ERR_CUDA;
     if (n == 0) {
         if ((flags & VOX_OUT_BITMASK) && (flags & VOX_OUT_FRESH) &&
             cudaMemsetAsync(d_mask, 0, 4 * static_cast<size_t>(vox_mask_words(dims)), s) != cudaSuccess)
@@ -1323,7 +1334,7 @@ vox_status vox_euclid_generate(const vox_segment *d_segs, int64_t n, vox_dims di
         return VOX_OK;
     }
     return launch_euclid(d_segs, n, dims, d_list, list_capacity, d_mask, flags, d_offsets, d_ws, ws_bytes, d_status, s,
-                         false);
+                         false, small);
 }
 
 vox_status vox_euclid_plan(const vox_segment *d_segs, int64_t n, vox_dims dims, void *d_ws, size_t ws_bytes,
@@ -1337,9 +1348,10 @@ vox_status vox_euclid_plan(const vox_segment *d_segs, int64_t n, vox_dims dims, 
     int64_t voxels = 0, samples = 0, pieces = 0;
     int32_t st = 0;
     if (n > 0) {
-        if (cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess) return VOX_ERR_CUDA;
+        const bool small = small_scan(n);
+        if (!small && cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess) return VOX_ERR_CUDA;
         if (vox_status e = launch_euclid(d_segs, n, dims, nullptr, 0, nullptr, 0, nullptr, d_ws, ws_bytes, d_status, s,
-                                         true))
+                                         true, small))
             return e;
         const EuclidLayout E = euclid_layout(n);
         const char *base = static_cast<const char *>(d_ws);

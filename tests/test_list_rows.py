@@ -71,3 +71,36 @@ def test_list_rows(name, bits):
         r = run_gpu(segs, (1024,) * 3, vox.OUT_LIST32 if bits == 32 else vox.OUT_LIST64, capacity=capacity)
         assert r["status"] == 0
         assert_list_equal(r["list_full"], want, len(want))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [1, 4095, 4096, 4097])  # one CTA's count + scan, and the tiled one
+def test_small_scan(n):
+    """Counts, offsets and list on both sides of the line between the two scans, with a
+    status word and a workspace that hold anything before the call; an endpoint outside."""
+    import torch
+
+    from gpu_util import get_oracle
+
+    rng = np.random.default_rng(n)
+    dims = (300, 200, 100)
+    segs = workloads.uniform_segments(rng, n, dims)
+    O = get_oracle()
+    want, off = O.list32(segs), np.concatenate([[0], np.cumsum(O.count(segs).astype(np.int64))])
+    d = torch.from_numpy(segs).cuda()
+    ws = torch.full((vox.vox_workspace_size(n),), 0xA5, dtype=torch.uint8, device="cuda")
+    status = torch.full((1,), 4, dtype=torch.int32, device="cuda")
+    counts = torch.empty(n, dtype=torch.int32, device="cuda")
+    offsets = torch.empty(n + 1, dtype=torch.int64, device="cuda")
+    vox.vox_count(d, dims, ws, status, counts, offsets)
+    assert int(status.item()) == 0
+    assert np.array_equal(offsets.cpu().numpy(), off) and np.array_equal(counts.cpu().numpy(), np.diff(off))
+    lst = torch.zeros(len(want), dtype=torch.int32, device="cuda")
+    ws.fill_(0x5A)
+    status.fill_(4)
+    vox.vox_generate(d, dims, ws, status, lst)
+    assert int(status.item()) == 0 and np.array_equal(lst.cpu().numpy().view(np.uint32), want)
+    d[n - 1, 5] = 100
+    lst.zero_()
+    vox.vox_generate(d, dims, ws, status, lst)
+    assert int(status.item()) == vox.ERR_OUT_OF_BOUNDS and int(lst.abs().sum()) == 0
