@@ -197,8 +197,8 @@ bool make_volume_tmap(const BrickGeom &G, uint32_t *mask, CUtensorMap *out, int3
 struct VolLayout {
     int64_t n_tiles;  // scan tiles over the brick counts
     size_t hdr;       // scan ticket at +0, number of brick parts at +64, brick ticket at +128
+    size_t desc;      // uint64 [n_tiles] (follows hdr: one memset resets both)
     size_t count;     // int32 [n_slots]
-    size_t desc;      // uint64 [n_tiles]
     size_t off;       // int64 [n_slots + 4]
     size_t cursor;    // int64 [n_slots + 1]
     size_t hot;       // HotPart [kHotParts]
@@ -213,8 +213,8 @@ struct EuclidLayout {
     int64_t n_runs;   // run slots
     int64_t n_tiles;  // scan tiles over the run counts
     size_t hdr;       // ticket of the run scan
+    size_t desc;      // uint64 [n_tiles] (follows hdr: one memset resets both)
     size_t count;     // int32 [n_runs]
-    size_t desc;      // uint64 [n_tiles]
     size_t off;       // int64 [n_runs + 4]
     size_t total;
 };
@@ -225,9 +225,9 @@ EuclidLayout euclid_layout(int64_t n)
     E.n_runs = std::max<int64_t>(n, kEuclidRunSlots);
     E.n_tiles = (E.n_runs + kScanTile - 1) / kScanTile;
     E.hdr = ws_layout(n).total;
-    E.count = E.hdr + kWsAlign;
-    E.desc = E.count + align_up(4 * static_cast<size_t>(E.n_runs));
-    E.off = E.desc + align_up(8 * static_cast<size_t>(E.n_tiles));
+    E.desc = E.hdr + kWsAlign;
+    E.count = E.desc + align_up(8 * static_cast<size_t>(E.n_tiles));
+    E.off = E.count + align_up(4 * static_cast<size_t>(E.n_runs));
     E.total = E.off + align_up(8 * static_cast<size_t>(E.n_runs + 4));
     return E;
 }
@@ -240,9 +240,9 @@ VolLayout vol_layout(int64_t n, const BrickGeom &G, int64_t capacity, size_t bas
     const size_t nb = static_cast<size_t>(G.n_slots);
     L.n_tiles = (G.n_slots + kScanTile - 1) / kScanTile;
     L.hdr = base != 0 ? base : ws_layout(n).total;
-    L.count = L.hdr + kWsAlign;
-    L.desc = L.count + align_up(4 * nb);
-    L.off = L.desc + align_up(8 * static_cast<size_t>(L.n_tiles));
+    L.desc = L.hdr + kWsAlign;
+    L.count = L.desc + align_up(8 * static_cast<size_t>(L.n_tiles));
+    L.off = L.count + align_up(4 * nb);
     L.cursor = L.off + align_up(8 * (nb + 4));
     L.hot = L.cursor + align_up(8 * (nb + 1));
     L.slopes = L.hot + align_up(sizeof(HotPart) * kHotParts);
@@ -489,8 +489,7 @@ vox_status launch_bricks(const vox_segment *segs, int64_t n, const BrickGeom &G,
     const VolLayout VL = vol_layout(n, G, 0, euclid ? euclid_layout(n).total : 0);
     const int64_t capacity = static_cast<int64_t>((ws_bytes - VL.pieces) / 8);
     char *base = static_cast<char *>(ws);
-    if (cudaMemsetAsync(base + VL.hdr, 0, kWsAlign, stream) != cudaSuccess) return VOX_ERR_CUDA;
-    if (cudaMemsetAsync(base + VL.desc, 0, VL.off - VL.desc, stream) != cudaSuccess) return VOX_ERR_CUDA;
+    if (cudaMemsetAsync(base + VL.hdr, 0, VL.count - VL.hdr, stream) != cudaSuccess) return VOX_ERR_CUDA;
     BinParams bp{};
     bp.segs = reinterpret_cast<const int32_t *>(segs);
     bp.n = n;
@@ -870,8 +869,7 @@ vox_status launch_euclid(const vox_segment *segs, int64_t n, vox_dims dims, void
     if (vox_status e = launch_count_scan(segs, n, dims, nullptr, nullptr, ws, ws_bytes, status, stream, nullptr,
                                          nullptr, 0, true, small))
         return e;
-    if (cudaMemsetAsync(base + E.hdr, 0, kWsAlign, stream) != cudaSuccess) return VOX_ERR_CUDA;
-    if (cudaMemsetAsync(base + E.desc, 0, E.off - E.desc, stream) != cudaSuccess) return VOX_ERR_CUDA;
+    if (cudaMemsetAsync(base + E.hdr, 0, E.count - E.hdr, stream) != cudaSuccess) return VOX_ERR_CUDA;
     EuclidParams p;
     p.segs = reinterpret_cast<const int32_t *>(segs);
     p.n = n;
