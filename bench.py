@@ -361,6 +361,165 @@ def aggregate_ranks(ms_local: float, voxels_local: int, world: int, device):
     return ms_max, total, total / (ms_max / 1000.0)
 
 
+# ------------------------------------------------------------ one scene's step
+class SceneBench:
+    """One scene's whole step (count + scan, the list, a fresh volume by bricks)
+    on resident buffers: tuned, timed eagerly phase by phase (events between
+    phases) and as batching.SceneStep (the same launches captured once as a CUDA
+    graph, list and volume on two streams), outputs checked equal."""
+
+    def __init__(self, key: str, w, list_flag: int, dev, tune: bool, tuning_arg: str = ""):
+        import torch
+
+        from paper_2009_09500_gb300 import vox
+
+        self.key, self.w, self.list_flag, self.dev = key, w, list_flag, dev
+        self.elem = 8 if list_flag == vox.OUT_LIST64 else 4
+        n = w.n
+        self.segs = torch.from_numpy(w.segs).to(dev)
+        self.status = torch.zeros(1, dtype=torch.int32, device=dev)
+        ws = torch.empty(vox.vox_workspace_size_volume(n, w.dims, 0), dtype=torch.uint8, device=dev)
+        self.V, self.P = vox.vox_plan(self.segs, w.dims, ws, self.status)
+        del ws
+        self.ws = torch.empty(vox.vox_workspace_size_volume(n, w.dims, self.P), dtype=torch.uint8, device=dev)
+        self.lst = torch.empty(self.V, dtype=torch.int64 if self.elem == 8 else torch.int32, device=dev)
+        self.words = vox.vox_mask_words(w.dims)
+        self.mask = torch.empty(self.words, dtype=torch.int32, device=dev)
+        self.flags = list_flag | vox.OUT_BITMASK | vox.OUT_FRESH
+        self.tuning = None
+        if tuning_arg:
+            knobs = [int(x) for x in tuning_arg.split(",")] + [0]
+            vox.vox_set_tuning(*knobs[:4])
+            self.tuning = {"params": vox.vox_get_tuning(), "given": True}
+        elif tune:
+            from paper_2009_09500_gb300 import autotune
+
+            self.tuning = autotune.get_or_tune(
+                lambda: vox.vox_generate(self.segs, w.dims, self.ws, self.status, self.lst, self.mask, self.flags),
+                n, self.V, w.dims, self.flags, reps=3)
+        else:
+            self.tuning = {"params": vox.vox_get_tuning()}
+
+    def step(self, s, ev=None):
+        from paper_2009_09500_gb300 import vox
+
+        w = self.w
+        if ev is not None:
+            ev[0].record(s)
+        vox.vox_count(self.segs, w.dims, self.ws, self.status, None, None, s)
+        if ev is not None:
+            ev[1].record(s)
+        vox.vox_generate_from_scan(self.segs, w.dims, self.ws, self.status, self.lst, None, self.list_flag, s,
+                                   capacity=self.V)
+        if ev is not None:
+            ev[2].record(s)
+        vox.vox_generate_from_scan(self.segs, w.dims, self.ws, self.status, None, self.mask,
+                                   vox.OUT_BITMASK | vox.OUT_FRESH, s)
+        if ev is not None:
+            ev[3].record(s)
+
+    def run(self, steps: int, warmup: int, flush, stream, world: int = 1, sampler=None) -> dict:
+        import torch
+
+        from paper_2009_09500_gb300 import batching, vox
+
+        for _ in range(warmup):
+            flush.zero_()
+            self.step(stream)
+        torch.cuda.synchronize()
+        self._check()
+        evs = [tuple(torch.cuda.Event(enable_timing=True) for _ in range(4)) for _ in range(steps)]
+        for k in range(steps):
+            flush.zero_()
+            self.step(stream, evs[k])
+        torch.cuda.synchronize()
+        self._check()
+        graph = batching.SceneStep(self.segs, self.w.dims, self.list_flag, volume=True, device=self.dev)
+        if (graph.V, graph.P) != (self.V, self.P):
+            raise RuntimeError("plan mismatch")
+        for _ in range(warmup):
+            flush.zero_()
+            graph.replay()
+        gevs = [tuple(torch.cuda.Event(enable_timing=True) for _ in range(2)) for _ in range(steps)]
+        if world > 1:
+            torch.distributed.barrier()
+        torch.cuda.synchronize()
+        if sampler is not None:
+            sampler.start()
+        t0 = time.perf_counter()
+        for k in range(steps):
+            flush.zero_()
+            gevs[k][0].record(stream)
+            graph.replay()
+            gevs[k][1].record(stream)
+        torch.cuda.synchronize()
+        wall = time.perf_counter() - t0
+        if world > 1:
+            torch.distributed.barrier()
+        clocks = sampler.stop() if sampler is not None else None
+        if int(graph.status.item()) != 0:
+            raise RuntimeError(f"device status {vox.strerror(int(graph.status.item()))}")
+        if not (torch.equal(graph.lst[:self.V], self.lst) and torch.equal(graph.mask, self.mask)):
+            raise RuntimeError("graph step and eager step disagree")
+        del graph
+        torch.cuda.empty_cache()
+        step_ms = [g[0].elapsed_time(g[1]) for g in gevs]
+        return {"step_ms": step_ms, "eager_ms": [e[0].elapsed_time(e[3]) for e in evs],
+                "count_ms": [e[0].elapsed_time(e[1]) for e in evs], "list_ms": [e[1].elapsed_time(e[2]) for e in evs],
+                "vol_ms": [e[2].elapsed_time(e[3]) for e in evs], "clocks": clocks, "wall_s": wall}
+
+    def _check(self):
+        from paper_2009_09500_gb300 import vox
+
+        st = int(self.status.item())
+        if st != 0:
+            raise RuntimeError(f"device status {vox.strerror(st)}")
+
+    def rooflines(self, t: dict, sms: int, mhz) -> dict:
+        """HBM rooflines of the list and volume phases (algorithmic bytes per
+        launch / mean eager phase time); `roofline` = the longer phase."""
+        peaks, peak_kind = _measured_peaks()
+        hbm = float(peaks["hbm_gbs"])
+        n = self.w.n
+        lname = "k_list<list64>" if self.elem == 8 else "k_list<list32>"
+        list_mean, vol_mean = float(np.mean(t["list_ms"])), float(np.mean(t["vol_ms"]))
+        list_bytes = 24 * n + self.elem * self.V
+        vol_bytes = 24 * n + 4 * self.words
+        vol_kernels = ["k_scan<false>", "k_bin_scatter", "k_brick_volume", "k_generate<volume, gated>"]
+        roof_list = {"bound": "hbm", "achieved": list_bytes / list_mean / 1e6, "peak": hbm, "unit": "GB/s",
+                     "frac": list_bytes / list_mean / 1e6 / hbm,
+                     "traffic": _recorded_field(self.key, [lname], "dram_bytes_per_launch"),
+                     "kernel": f"{lname} (one launch)", "peak_kind": f"{peak_kind} HBM copy",
+                     "algorithmic_bytes_per_launch": list_bytes, "ms": list_mean,
+                     "bytes_model": f"24 B/segment read + {self.elem} B/voxel written",
+                     "issue": _issue(self.key, [lname], list_mean, mhz, sms)}
+        roof_vol = {"bound": "hbm", "achieved": vol_bytes / vol_mean / 1e6, "peak": hbm, "unit": "GB/s",
+                    "frac": vol_bytes / vol_mean / 1e6 / hbm,
+                    "traffic": _recorded_field(self.key, vol_kernels, "dram_bytes_per_launch"),
+                    "kernel": "volume phase: k_scan<false> + k_bin_scatter + k_brick_volume (one TMA tensor store "
+                              "per brick) + gated atomic fallback (exits at once); k_bin_count runs in the count phase",
+                    "peak_kind": f"{peak_kind} HBM copy", "algorithmic_bytes_per_launch": vol_bytes, "ms": vol_mean,
+                    "bytes_model": "24 B/segment read + the whole volume written once (w*h*d/8 bytes)",
+                    "pieces": self.P, "issue": _issue(self.key, vol_kernels, vol_mean, mhz, sms)}
+        return (roof_vol, roof_list) if vol_mean >= list_mean else (roof_list, roof_vol)
+
+    def summary(self, t: dict) -> dict:
+        step = t["step_ms"]
+        ms = float(np.mean(step))
+        return {"segments": self.w.n, "voxels": self.V, "pieces": self.P, "ms_per_step": ms,
+                "voxels_per_s": self.V / ms * 1e3, "segments_per_s": self.w.n / ms * 1e3,
+                "p50_ms": float(np.percentile(step, 50)), "p99_ms": float(np.percentile(step, 99)),
+                "kernels_ms": {"count_scan": float(np.mean(t["count_ms"])), "list": float(np.mean(t["list_ms"])),
+                               "volume": float(np.mean(t["vol_ms"]))},
+                "eager_ms_per_step": float(np.mean(t["eager_ms"])), "tuning": self.tuning}
+
+    def free(self):
+        import torch
+
+        del self.segs, self.ws, self.lst, self.mask
+        torch.cuda.empty_cache()
+
+
 def measure_e2e(w, list_flag: int, P: int, reps: int, dev, stream) -> dict:
     """End to end through vox_generate_host: pinned host segments in, the list
     and the fresh volume out to pinned host buffers, all inside the timed call."""
@@ -938,7 +1097,8 @@ def run_ours(args):
         "roofline": roofline, "roofline_other": roofline_other, "cpu_baseline": cpu, "cpu_baseline_all_cores": cpu_all,
         "e2e": e2e, "clocks": clocks,
         "gpu_launches": 7 * args.steps,
-        "gpu_launches_note": "graph-timed region, per step: k_scan<true>, k_bin_count, k_list, k_scan<false>, k_bin_scatter, k_brick_volume, "
+        "gpu_launches_note": "graph-timed region, per step: k_scan<true>, k_bin_count, k_list, k_scan<false>, "
+                             "k_bin_scatter, k_brick_volume, "
                              "k_generate (gated volume fallback; exits at once); the eager per-phase region launches "
                              "the same 7 per step",
         "batched_vs_plain": batched, "config2_fixed_length": cfg2, "config1_latency": latency,
