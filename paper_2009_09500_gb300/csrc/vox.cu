@@ -251,6 +251,16 @@ VolLayout vol_layout(int64_t n, const BrickGeom &G, int64_t capacity, size_t bas
     return L;
 }
 
+// G with the slots that any volume (or batch) of at most as many bricks takes: fewer
+// bricks have more counter replicas, and a workspace sized for the larger volume serves
+// the smaller one too.
+BrickGeom slots_up_to(BrickGeom G, bool batch)
+{
+    for (const int64_t nb : {int64_t(kBricks32Replicas), batch ? int64_t(kBricks8Replicas) : int64_t(0)})
+        if (G.n_bricks > nb) G.n_slots = std::max(G.n_slots, nb * kPieceClasses * counter_replicas(nb));
+    return G;
+}
+
 // Whether a call on n segments with this workspace builds the volume by brick
 // ownership (the workspace holds the brick arrays and room for a piece).
 // Pieces name their segment in 32 bits: beyond 2^32 segments the volume takes
@@ -1199,7 +1209,8 @@ size_t vox_workspace_size_batched_volume(int64_t n_total, int32_t n_scenes, int6
 {
     if (n_total < 0 || n_scenes < 1 || total_bricks < 0 || piece_capacity < 0) return 0;
     if (total_bricks == 0) return batch_layout(n_total, n_scenes).total;
-    return batch_brick_layout(n_total, n_scenes, total_bricks, piece_capacity > 0 ? piece_capacity : 1).VL.total;
+    const BatchBrickLayout L = batch_brick_layout(n_total, n_scenes, total_bricks, 0);
+    return vol_layout(n_total, slots_up_to(L.tot, true), piece_capacity > 0 ? piece_capacity : 1, L.VL.hdr).total;
 }
 
 vox_status vox_plan_batched(const vox_segment *d_segs, int64_t n_total, const vox_scene *d_scenes, int32_t n_scenes,
@@ -1307,7 +1318,7 @@ size_t vox_euclid_workspace_size_volume(int64_t n, vox_dims dims, int64_t piece_
     BrickGeom G;
     const size_t base = euclid_layout(n).total;
     if (!make_geom(dims, &G)) return base;
-    return vol_layout(n, G, piece_capacity > 0 ? piece_capacity : 1, base).total;
+    return vol_layout(n, slots_up_to(G, false), piece_capacity > 0 ? piece_capacity : 1, base).total;
 }
 
 vox_status vox_euclid_generate(const vox_segment *d_segs, int64_t n, vox_dims dims, void *d_list,
@@ -1379,7 +1390,7 @@ size_t vox_workspace_size_volume(int64_t n, vox_dims dims, int64_t piece_capacit
     if (n < 0 || piece_capacity < 0) return 0;
     BrickGeom G;
     if (!make_geom(dims, &G)) return ws_layout(n).total;
-    return vol_layout(n, G, piece_capacity > 0 ? piece_capacity : 1).total;
+    return vol_layout(n, slots_up_to(G, false), piece_capacity > 0 ? piece_capacity : 1).total;
 }
 
 vox_status vox_plan(const vox_segment *d_segs, int64_t n, vox_dims dims, void *d_ws, size_t ws_bytes,

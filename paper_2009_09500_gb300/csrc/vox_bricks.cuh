@@ -12,10 +12,12 @@
 // volume sector then crosses DRAM at most twice (read + write), whatever the
 // number of voxels in it.
 //
-//   k_bin_count    pieces per brick (lanes walk segments' pieces, global atomics)
-//   k_scan<false>  exclusive scan of the per-brick counts (decoupled look-back)
-//   k_bin_scatter  pieces written into their brick's bucket
-//   k_brick_volume one CTA per brick: voxels -> shared bitmap -> volume
+//   k_bin_count    pieces per slot of a brick (lanes walk segments' pieces, global atomics)
+//   k_scan<false>  exclusive scan of the slot counts (decoupled look-back)
+//   k_bin_scatter  pieces written into their slot; the segments' slope table
+//   k_brick_volume one CTA per brick, or part of one with very many pieces: voxels ->
+//                  shared bitmap -> volume
+//   k_unbrick_tma  brick-major volume -> row-major volume
 //
 // A piece is (segment, first step k, length). The steps at which a segment's
 // coordinate on an axis enters the next brick follow from the same exact rounding
@@ -71,9 +73,14 @@ constexpr int64_t kMaxBricks = int64_t(1) << 26;
 // it, and updates of one address go one after another, so few bricks get more of them.
 // Binning of 48 scenes (1.17 M segments, 1,623 bricks in all), one counter per (brick,
 // class): 128 + 110 us (scatter, count), eight: 104 + 62 us.
+// More of them cost the slot scan what the counting gains (48 scenes with 32: 46 instead
+// of 60 us of counting, 15 instead of 7 us of scanning).
+constexpr int32_t kBricks32Replicas = 512;
+constexpr int32_t kBricks8Replicas = 32768;
+
 __host__ __device__ inline int32_t counter_replicas(int64_t bricks)
 {
-    return bricks <= 512 ? 32 : (bricks <= 32768 ? 8 : 1);
+    return bricks <= kBricks32Replicas ? 32 : (bricks <= kBricks8Replicas ? 8 : 1);
 }
 
 // Brick shape for a volume whose rows are whole 32-bit words (w % 32 == 0):
@@ -941,13 +948,14 @@ __device__ __forceinline__ void take_brick(const BrickParams &p, bool overflow, 
     }
 }
 
-// One CTA per brick, or part of a brick (HotPart; dynamic tickets, the parts first, taken two bricks ahead by the last warp
-// while the others walk, so that no barrier waits for a ticket). The brick's
+// One CTA per brick, or part of a brick (HotPart; dynamic tickets, the parts first, taken
+// two bricks ahead by the last warp while the others walk, so that no barrier waits for
+// a ticket). The brick's
 // pieces arrive ordered by length class, longest first (the bucket order of the
 // binning). Group w of 32 consecutive pieces goes to warp w, further groups to
 // the warps that ask a shared counter first: the lanes of a warp walk pieces of
-// similar length (at most kPieceMaxLen steps), longest groups first. A warp's
-// A warp's first group of the next brick is loaded while it walks the current one
+// similar length (at most kPieceMaxLen steps), longest groups first. A
+// warp's first group of the next brick is loaded while it walks the current one
 // (its pieces during the walk, their segments' slopes after it), so that, with
 // about as many groups per brick as warps, most groups start without waiting
 // for global memory. Each lane enters its piece's segment at the piece's first

@@ -1,14 +1,17 @@
-// vox_kernels.cuh -- the three kernels of the voxelization hot path (sm_103a):
+// vox_kernels.cuh -- the scans and the voxel-range generation (sm_103a):
 //
 //   k_scan        per-segment voxel count N + 1 (+ endpoint validation) fused
 //                 with a single-pass decoupled look-back exclusive scan
 //                 (Merrill & Garland, 2016) into int64 offsets;
-//   k_generate    voxel-parallel generation: each CTA owns a contiguous range of
-//                 global voxel ids, stages windows of segment records and offsets
-//                 into shared memory with 1-D TMA bulk copies, maps each thread's
-//                 run of R voxels back to (segment, k) by a search in the staged
-//                 offsets, and steps through the run with the exact integer
-//                 recurrence, writing packed coordinates and/or OR-ing bits.
+//   k_scan_small  the same for at most 4096 segments, by one CTA;
+//   k_generate    volumes by per-voxel atomics (with or without the list in the
+//                 same pass): each CTA owns a contiguous range of global voxel
+//                 ids, stages windows of segment records and offsets into shared
+//                 memory with 1-D TMA bulk copies, maps each thread's run of R
+//                 voxels back to (segment, k) by a search in the staged offsets,
+//                 and steps through the run with the exact integer recurrence,
+//                 writing packed coordinates and OR-ing bits. The list alone is
+//                 k_list's (vox_list.cuh).
 //
 // The paper's multi-segment kernel pads every segment to N_max threads (Section 5,
 // Fig. 4b) and names the resulting divergence as its main loss for segments of

@@ -59,8 +59,9 @@ class ServeRequest:
 
     @property
     def device_bytes(self) -> int:
-        """Volume + segments + workspace share (with brick pieces) of this request."""
-        return self.mask_bytes + 24 * self.n + 16 * self.n + 8 * self.piece_capacity + 256
+        """Volume + segments + workspace share (scan, 32-byte slopes and brick pieces)
+        of this request."""
+        return self.mask_bytes + 24 * self.n + (16 + 32) * self.n + 8 * self.piece_capacity + 256
 
     @property
     def latency_ms(self) -> float:

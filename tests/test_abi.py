@@ -82,3 +82,18 @@ def test_brick_shape_queries(lib):
     assert vox.vox_mask_words_bricked((13, 7, 5)) == 0
     with pytest.raises(vox.VoxError):
         vox.vox_brick_shape((13, 7, 5))
+
+
+def test_workspace_serves_fewer_bricks(lib):
+    # counter replicas change at 512 and 32768 bricks: a workspace sized for more bricks
+    # (or more segments) is never too small for fewer
+    from paper_2009_09500_gb300 import vox
+
+    around = (1, 511, 512, 513, 600, 2047, 2048, 2049)
+    for size in (vox.vox_workspace_size_volume, vox.vox_euclid_workspace_size_volume):
+        for n in (1, 5000):
+            sizes = [size(n, (256, 64 * nb, 64), 100) for nb in around]  # nb bricks
+            assert sizes == sorted(sizes)
+    sizes = [vox.vox_workspace_size_batched_volume(5000, 3, nb, 100)
+             for nb in around + (32767, 32768, 32769, 262143, 262144, 262145)]
+    assert sizes == sorted(sizes)
