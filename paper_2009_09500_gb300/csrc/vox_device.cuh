@@ -358,9 +358,9 @@ struct EuclidStepper {
         L = static_cast<LinT>(v[0]) + static_cast<LinT>(v[1]) * w + static_cast<LinT>(v[2]) * wh;
     }
 
-    // Advance one sample; true when the voxel changed (some axis moved).
+    // Advance one sample; 1 when the voxel changed (some axis moved), else 0.
     template <bool kP, bool kL>
-    __device__ __forceinline__ bool step()
+    __device__ __forceinline__ uint32_t step()
     {
         uint32_t c[3];
 #pragma unroll
@@ -370,7 +370,7 @@ struct EuclidStepper {
         }
         if (kP) P += static_cast<PackT>(c[0]) * dP[0] + static_cast<PackT>(c[1]) * dP[1] + static_cast<PackT>(c[2]) * dP[2];
         if (kL) L += static_cast<LinT>(c[0]) * dL[0] + static_cast<LinT>(c[1]) * dL[1] + static_cast<LinT>(c[2]) * dL[2];
-        return (c[0] | c[1] | c[2]) != 0u;
+        return c[0] | c[1] | c[2];
     }
 };
 

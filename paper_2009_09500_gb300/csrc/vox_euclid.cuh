@@ -170,23 +170,39 @@ __global__ void __launch_bounds__(256) k_euclid_runs(EuclidParams p)
 // segment: at the top of each pass every lane that needs one enters its next
 // segment (one division per axis, taken by the lanes together rather than each
 // at its own step), then walks the part in a tight loop. A lane stops when it is
-// done, its next segment lies beyond the window, or (list) its row is full; when
-// every lane has stopped, full rows are flushed and the walk goes on in the same
-// window, else the window moves on. Count pass: the voxels each run adds (run_count).
-// List pass: each lane appends its voxels to its own row of the warp's stage
-// (32 entries for 32-bit lists, 16 for 64-bit ones, rows padded by one entry so
-// that lanes at equal fill hit different banks), and a flush writes every row,
-// row by row, with coalesced stores at the rows' list positions. Segment offsets
-// and (optionally) the volume's atomics are written on the way.
-template <typename PackT>
-__host__ __device__ constexpr int euclid_row() { return sizeof(PackT) == 4 ? 32 : 16; }
+// done, its next segment lies beyond the window, (list) its row is full, or after
+// kPart samples while some lane's part is shorter; when every lane has stopped, full
+// rows are flushed and the walk goes on in the same window, else the window moves on.
+// Count pass: the voxels each run adds (run_count).
+// List pass: each lane appends its voxels to its own row of the warp's stage (rows
+// padded by one entry so that lanes at equal fill hit different banks), and a flush
+// writes every row with coalesced stores at the rows' list positions, which the lanes
+// leave in shared memory so that a row costs one 16-byte load instead of three
+// shuffles. Segment offsets and (optionally) the volume's atomics are written on the way.
+// Bound by instruction issue. List pass, us, before and after the rows' positions in
+// shared memory with eight rows in flight, 32 entries a row for 64-bit lists too, and
+// passes that end for the shortest part: 1M segments of 64 steps, 32-bit 230 -> 176;
+// 200,000 uniform segments, 64-bit 252 -> 164; 10^8 voxels in 1024 segments 433 -> 294;
+// 1M segments of 6 steps 87 -> 75. Count pass: 113 -> 102, 77 -> 76, 80 -> 78, 54 -> 53.
+// Rows of 64 entries: 211 us on the first (fewer
+// warps). Windows of 32 segments: 250 + 152 us; of 128: 189 + 115 (but 58 + 41 instead
+// of 74 + 52 on 1M segments of 6 steps). Parts of 12, 16, 24, 28 samples in the list
+// pass: 182, 177, 177, 182; of 16, 24, 32 in the count pass: 108, 102, 104.
+// With the volume's atomics a 64-bit row of 32 entries costs more warps than it gains
+// (195 against 180 us on 100,000 segments in 555 x 206 x 645).
+template <typename PackT, bool kMask>
+__host__ __device__ constexpr int euclid_row() { return sizeof(PackT) == 8 && kMask ? 16 : 32; }
 
-// Largest j in [0, cnt) with offs[j] <= r, given offs[0] <= r < offs[cnt], cnt <= 64.
+constexpr int kEuclidWin = 64;        // segments per staged window
+constexpr int kEuclidListPart = 20;   // samples of a pass while some lane's part is shorter
+constexpr int kEuclidCountPart = 40;
+
+// Largest j in [0, cnt) with offs[j] <= r, given offs[0] <= r < offs[cnt], cnt <= kEuclidWin.
 __device__ __forceinline__ int32_t find_in_window64(const int64_t *offs, int32_t cnt, int64_t r)
 {
     int32_t lo = 0;
 #pragma unroll
-    for (int32_t step = 32; step > 0; step >>= 1) {
+    for (int32_t step = kEuclidWin / 2; step > 0; step >>= 1) {
         const int32_t m = lo + step;
         if (m < cnt && offs[m] <= r) lo = m;
     }
@@ -194,25 +210,34 @@ __device__ __forceinline__ int32_t find_in_window64(const int64_t *offs, int32_t
 }
 
 constexpr int kEuclidWarps = 4;  // warps per CTA of the warp walk
-constexpr int kEuclidWin = 64;   // segments per staged window
 
-template <typename PackT, bool kRows>
+template <typename PackT, bool kRows, bool kMask>
 struct EuclidWarpSmem {
     int64_t offs[kEuclidWin + 1];  // sample offsets of the window's segments (+ the next)
     int32_t recs[kEuclidWin * 6];  // the window's segment records
-    PackT rows[kRows ? 32 * (euclid_row<PackT>() + 1) : 1];
+    uint4 head[kRows ? 32 : 1];    // at a flush: where each row goes, and its entries
+    PackT rows[kRows ? 32 * (euclid_row<PackT, kMask>() + 1) : 1];
 };
 
+// CTAs per SM asked of the compiler: the list with the volume's atomics runs faster in
+// fewer registers (100,000 segments in 555 x 206 x 645, 64-bit list and volume 178 -> 169 us), the
+// list alone does not (200,000 uniform segments 179 -> 183).
+template <bool kWrite, int OUT>
+__host__ __device__ constexpr int euclid_ctas() { return !kWrite ? 12 : (OUT & kOutMask) != 0 ? 7 : 1; }
+
 template <bool kWrite, int OUT, bool LIN64>
-__global__ void __launch_bounds__(32 * kEuclidWarps, kWrite ? 1 : 12) k_euclid_warp(EuclidParams p)
+__global__ void __launch_bounds__(32 * kEuclidWarps, euclid_ctas<kWrite, OUT>()) k_euclid_warp(EuclidParams p)
 {
     using PackT = typename std::conditional<(OUT & kOutList64) != 0, uint64_t, uint32_t>::type;
     using LinT = typename std::conditional<LIN64, uint64_t, uint32_t>::type;
     constexpr bool kList = kWrite && (OUT & (kOutList32 | kOutList64)) != 0;
     constexpr bool kMask = kWrite && (OUT & kOutMask) != 0;
-    constexpr int kRow = euclid_row<PackT>();
+    constexpr int kRow = euclid_row<PackT, kMask>();
     constexpr int kStride = kRow + 1;
-    using Smem = EuclidWarpSmem<PackT, kList>;
+    constexpr int kRowsAtOnce = kRow < 32 ? 32 / kRow : 1;
+    constexpr int kFlushUnroll = 8;
+    constexpr int kPart = kList ? kEuclidListPart : kEuclidCountPart;
+    using Smem = EuclidWarpSmem<PackT, kList, kMask>;
     __shared__ Smem smem_all[kEuclidWarps];
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
@@ -245,7 +270,7 @@ __global__ void __launch_bounds__(32 * kEuclidWarps, kWrite ? 1 : 12) k_euclid_w
             int32_t i = 0;
             int32_t i_end = 0;     // end of the current segment, as a sample index of the run
             bool in_seg = false;   // stepping state valid for the current segment
-            bool add = false;      // the current sample adds its voxel
+            uint32_t add = 0;      // 1 where the current sample adds its voxel
             int64_t cur = 0;       // the current segment
             EuclidStepper<PackT, LinT> st;
             int64_t outp = (kWrite && has && (kList || p.seg_off != nullptr)) ? __ldg(p.run_off + j) : 0;
@@ -253,12 +278,20 @@ __global__ void __launch_bounds__(32 * kEuclidWarps, kWrite ? 1 : 12) k_euclid_w
             LinT cur_word = static_cast<LinT>(~LinT(0));
             uint32_t acc = 0;
             auto flush = [&]() {
+                const uint64_t at = reinterpret_cast<uint64_t>(list + outp);
+                sm.head[lane] = make_uint4(static_cast<uint32_t>(at), static_cast<uint32_t>(at >> 32),
+                                           static_cast<uint32_t>(f), 0u);
                 __syncwarp();
-#pragma unroll 1
-                for (int l = 0; l < 32; ++l) {
-                    const int fl = __shfl_sync(0xffffffffu, f, l);
-                    const int64_t ol = __shfl_sync(0xffffffffu, outp, l);
-                    if (lane < fl) list[ol + lane] = sm.rows[l * kStride + lane];
+#pragma unroll kFlushUnroll
+                for (int l = 0; l < 32; l += kRowsAtOnce) {
+                    const int r = l + lane / kRow;  // lane / kRow: 0 where a row takes the whole warp
+                    const uint4 h = sm.head[r];
+                    PackT *const to = reinterpret_cast<PackT *>(static_cast<uint64_t>(h.x) | static_cast<uint64_t>(h.y) << 32);
+#pragma unroll
+                    for (int c = 0; c < kRow; c += 32) {
+                        const int u = c + lane % kRow;
+                        if (u < static_cast<int>(h.z)) to[u] = sm.rows[r * kStride + u];
+                    }
                 }
                 __syncwarp();
                 outp += f;
@@ -288,7 +321,7 @@ __global__ void __launch_bounds__(32 * kEuclidWarps, kWrite ? 1 : 12) k_euclid_w
                         const int32_t *rec = sm.recs + 6 * jj;
                         if (k0 == 0) {
                             st.enter_n(rec, N, 0, w, wh);
-                            add = true;
+                            add = 1;
                             // the segment's first voxel lands at the lane's next output
                             // position (a flush moves outp and f together)
                             if (kWrite && p.seg_off != nullptr) p.seg_off[cur] = outp + f;
@@ -299,6 +332,9 @@ __global__ void __launch_bounds__(32 * kEuclidWarps, kWrite ? 1 : 12) k_euclid_w
                         in_seg = true;
                     }
                     int32_t m = in_seg ? i_end - i : 0;  // samples left in this segment part
+                    // while some lane's part ends soon, the others stop too, so that it
+                    // can enter its next segment
+                    if (__any_sync(0xffffffffu, in_seg && m < kPart)) m = min(m, kPart);
                     if constexpr (kList) m = min(m, kRow - f);  // one row entry per sample at most
                     // the next sample's flag comes from each step (a step past the
                     // segment's end is discarded: the next segment is entered afresh)
@@ -323,13 +359,13 @@ __global__ void __launch_bounds__(32 * kEuclidWarps, kWrite ? 1 : 12) k_euclid_w
 #pragma unroll 4
                         for (int32_t e = 0; e < m; ++e) {
                             row[f] = st.P;
-                            f += add ? 1 : 0;
+                            f += static_cast<int32_t>(add);
                             add = st.template step<kList, kMask>();
                         }
                     } else {
 #pragma unroll 4
                         for (int32_t e = 0; e < m; ++e) {
-                            cnt += add ? 1 : 0;
+                            cnt += static_cast<int32_t>(add);
                             add = st.template step<kList, kMask>();
                         }
                     }

@@ -198,3 +198,16 @@ def test_long_runs_many_row_flushes():
     segs = workloads._segments_from_major(rng, np.full(2000, 99_999, np.int64), edge).astype(np.int32)
     r = check(segs, (edge, edge, edge), L64)
     assert r["Vd"] > 2000 * 100_000
+
+
+@pytest.mark.parametrize("flags", [L32, L64, L32 | BM, L64 | BM])
+@pytest.mark.parametrize("edge", [16, 64, 600])
+def test_rows_and_parts(flags, edge):
+    """Segment parts and rows at their lengths' edges: equal lengths around a pass (20
+    and 40 samples), a row (16 and 32 entries) and a window (64 segments), then all of
+    them mixed with points and long segments."""
+    rng = np.random.default_rng(edge)
+    lengths = [v for v in (1, 2, 15, 16, 17, 19, 20, 21, 31, 32, 33, 39, 40, 41, 64, 65, 599) if v <= edge]
+    parts = [workloads.sweep_fixed(v, n=129, edge=edge).segs for v in lengths]
+    for segs in [parts[0], parts[-1], rng.permutation(np.concatenate(parts))]:
+        check(np.ascontiguousarray(segs), (edge,) * 3, flags)
