@@ -274,27 +274,25 @@ int grid_ctas(const void *kernel, int threads, size_t smem);
 
 // The binning passes: persistent grids (SMs x CTAs per SM, no more CTAs than
 // the segments fill), warps taking batches of segments.
-template <bool kEuclid, bool kBatched, int kPer>
-vox_status launch_bin_p(const BinParams &bp, bool scatter, int64_t n, cudaStream_t stream)
+template <int kPer>
+vox_status launch_bin_grid(void (*k)(BinParams), const BinParams &bp, int64_t n, cudaStream_t stream)
 {
-    const void *k = scatter ? reinterpret_cast<const void *>(k_bin_scatter<kEuclid, kBatched, kPer>)
-                            : reinterpret_cast<const void *>(k_bin_count<kEuclid, kBatched, kPer>);
-    int grid = grid_ctas(k, kBinThreads, 0);
+    int grid = grid_ctas(reinterpret_cast<const void *>(k), kBinThreads, 0);
     if (grid <= 0) return VOX_ERR_CUDA;
     constexpr int kCta = kBinWarps * 32 * kPer;  // segments of a CTA's first batches
     grid = static_cast<int>(std::min<int64_t>(grid, (n + kCta - 1) / kCta));
-    if (scatter) k_bin_scatter<kEuclid, kBatched, kPer><<<static_cast<unsigned>(grid), kBinThreads, 0, stream>>>(bp);
-    else k_bin_count<kEuclid, kBatched, kPer><<<static_cast<unsigned>(grid), kBinThreads, 0, stream>>>(bp);
+    k<<<static_cast<unsigned>(grid), kBinThreads, 0, stream>>>(bp);
     return cudaGetLastError() == cudaSuccess ? VOX_OK : VOX_ERR_CUDA;
 }
 
-// Segments per lane and batch: four when that leaves every warp of the grid about a
-// batch (4,864 warps), else two (the figures at bin_loop).
+// Segments per lane and batch (the figures at bin_loop): two to scatter, and to count
+// until four leave every warp of the grid about two batches.
 template <bool kEuclid, bool kBatched>
 vox_status launch_bin_t(const BinParams &bp, bool scatter, int64_t n, cudaStream_t stream)
 {
-    return n >= (int64_t(1) << 18) ? launch_bin_p<kEuclid, kBatched, 4>(bp, scatter, n, stream)
-                                   : launch_bin_p<kEuclid, kBatched, 2>(bp, scatter, n, stream);
+    if (scatter) return launch_bin_grid<2>(k_bin_scatter<kEuclid, kBatched, 2>, bp, n, stream);
+    return n > (int64_t(1) << 20) ? launch_bin_grid<4>(k_bin_count<kEuclid, kBatched, 4>, bp, n, stream)
+                                  : launch_bin_grid<2>(k_bin_count<kEuclid, kBatched, 2>, bp, n, stream);
 }
 
 vox_status launch_bin(const BinParams &bp, bool euclid, bool batched, bool scatter, int64_t n, cudaStream_t stream)

@@ -413,14 +413,17 @@ __device__ __forceinline__ void load_record(const int32_t *segs, int64_t s, int3
 // updates/s), else by the walk's instructions. Counting + scattering pass, us, against
 // a lane per segment in batches of 128 sorted by octave, with a branch per axis at
 // every run's end and four reservations in flight:
-//   4M log-uniform segments, 4096^3 (57 M pieces)   461 + 1295 -> 415 + 1075
-//   1M log-uniform segments, 2048^3                  73 +  222 ->  79 +  162
-//   48 uneven scenes (1.17 M segments)              132 +  196 ->  60 +  112
+//   4M log-uniform segments, 4096^3 (57 M pieces)   461 + 1295 -> 415 + 1072
+//   1M log-uniform segments, 2048^3                  73 +  222 ->  83 +  187
+//   48 uneven scenes (1.17 M segments)              132 +  196 ->  59 +  100
 //   200,000 uniform segments, 512^3                  35 +   50 ->  22 +   30
 //   1,000 uniform segments, 512 x 300 x 200          13 +   33 ->   7 +   13
 // kPer segments per lane and batch: more of them fill the rounds of equal octaves
-// better (4M: 444 + 1072 with 2, 653 + 1191 with 1), fewer keep more warps busy (the
-// 200,000: 26 + 38 with 4); launch_bin_t draws the line at 2^18 segments.
+// better, fewer keep more warps busy. Counting + scattering with four and two: 48 uneven
+// scenes 59 + 110 and 65 + 100; 5 scenes of 1.3 M segments 161 + 241 and 157 + 203; 1M
+// segments of 64 voxels 27 + 51 and 24 + 49, 3M 67 + 147 and 68 + 138; log-uniform 260,000
+// 14 + 31 and 14 + 26, 1M 80 + 177 and 83 + 187, 3M 326 + 859 and 347 + 839 (4M with one:
+// 653 + 1191). launch_bin_t takes two, and four to count more than 2^20 segments.
 // A lane per piece, its step and brick found by fixed-point slopes, takes about 300
 // instructions a piece (779 + 1128 us on the first).
 constexpr int kBinThreads = 256;
