@@ -496,8 +496,8 @@ class SceneBench:
         roof_vol = {"bound": "hbm", "achieved": vol_bytes / vol_mean / 1e6, "peak": hbm, "unit": "GB/s",
                     "frac": vol_bytes / vol_mean / 1e6 / hbm,
                     "traffic": _recorded_field(self.key, vol_kernels, "dram_bytes_per_launch"),
-                    "kernel": "volume phase: k_scan<false> + k_bin_scatter + k_brick_volume (one TMA tensor store "
-                              "per brick) + gated atomic fallback (exits at once); k_bin_count runs in the count phase",
+                    "kernel": "volume phase: k_scan<false> + k_bin_scatter + k_brick_volume (a TMA tensor store "
+                              "per quarter brick) + gated atomic fallback (exits at once); k_bin_count runs in the count phase",
                     "peak_kind": f"{peak_kind} HBM copy", "algorithmic_bytes_per_launch": vol_bytes, "ms": vol_mean,
                     "bytes_model": "24 B/segment read + the whole volume written once (w*h*d/8 bytes)",
                     "pieces": self.P, "issue": _issue(self.key, vol_kernels, vol_mean, mhz, sms)}
@@ -663,7 +663,7 @@ def measure_batched(steps: int, dev, tune: bool = True) -> dict:
         "batched_eager_ms": batched_eager[0], "plain_eager_ms": plain_eager[0],
         "batched_over_plain_eager": plain_eager[0] / batched_eager[0],
         "launches": {"batched": "one sequence: scene map, count + scan, scene bases, list, scene bricks, bin count, "
-                                "slot scan, scatter, brick volume, gated atomics (10 kernels + 3 memsets)",
+                                "slot scan, scatter, brick volume, gated atomics (10 kernels + memsets)",
                      "plain": "per scene: 2-3 memsets + 7 kernels (256 scenes)"},
         "tuning": tuning["params"],
     }
