@@ -253,10 +253,11 @@ VolLayout vol_layout(int64_t n, const BrickGeom &G, int64_t capacity, size_t bas
 
 // G with the slots that any volume (or batch) of at most as many bricks takes: fewer
 // bricks have more counter replicas, and a workspace sized for the larger volume serves
-// the smaller one too.
-BrickGeom slots_up_to(BrickGeom G, bool batch)
+// the smaller one too (beyond 32768 bricks, volumes of 4 GiB and more, that is the room
+// of 32768 bricks with eight replicas).
+BrickGeom slots_up_to(BrickGeom G)
 {
-    for (const int64_t nb : {int64_t(kBricks32Replicas), batch ? int64_t(kBricks8Replicas) : int64_t(0)})
+    for (const int64_t nb : {int64_t(kBricks32Replicas), int64_t(kBricks8Replicas)})
         if (G.n_bricks > nb) G.n_slots = std::max(G.n_slots, nb * kPieceClasses * counter_replicas(nb));
     return G;
 }
@@ -1208,7 +1209,7 @@ size_t vox_workspace_size_batched_volume(int64_t n_total, int32_t n_scenes, int6
     if (n_total < 0 || n_scenes < 1 || total_bricks < 0 || piece_capacity < 0) return 0;
     if (total_bricks == 0) return batch_layout(n_total, n_scenes).total;
     const BatchBrickLayout L = batch_brick_layout(n_total, n_scenes, total_bricks, 0);
-    return vol_layout(n_total, slots_up_to(L.tot, true), piece_capacity > 0 ? piece_capacity : 1, L.VL.hdr).total;
+    return vol_layout(n_total, slots_up_to(L.tot), piece_capacity > 0 ? piece_capacity : 1, L.VL.hdr).total;
 }
 
 vox_status vox_plan_batched(const vox_segment *d_segs, int64_t n_total, const vox_scene *d_scenes, int32_t n_scenes,
@@ -1316,7 +1317,7 @@ size_t vox_euclid_workspace_size_volume(int64_t n, vox_dims dims, int64_t piece_
     BrickGeom G;
     const size_t base = euclid_layout(n).total;
     if (!make_geom(dims, &G)) return base;
-    return vol_layout(n, slots_up_to(G, false), piece_capacity > 0 ? piece_capacity : 1, base).total;
+    return vol_layout(n, slots_up_to(G), piece_capacity > 0 ? piece_capacity : 1, base).total;
 }
 
 vox_status vox_euclid_generate(const vox_segment *d_segs, int64_t n, vox_dims dims, void *d_list,
@@ -1388,7 +1389,7 @@ size_t vox_workspace_size_volume(int64_t n, vox_dims dims, int64_t piece_capacit
     if (n < 0 || piece_capacity < 0) return 0;
     BrickGeom G;
     if (!make_geom(dims, &G)) return ws_layout(n).total;
-    return vol_layout(n, slots_up_to(G, false), piece_capacity > 0 ? piece_capacity : 1).total;
+    return vol_layout(n, slots_up_to(G), piece_capacity > 0 ? piece_capacity : 1).total;
 }
 
 vox_status vox_plan(const vox_segment *d_segs, int64_t n, vox_dims dims, void *d_ws, size_t ws_bytes,
