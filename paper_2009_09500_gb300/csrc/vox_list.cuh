@@ -45,11 +45,10 @@ constexpr int kListWarps = 8;                  // warps per CTA
 constexpr int kListThreads = 32 * kListWarps;
 constexpr int kListCtas = 4;                   // CTAs per SM
 constexpr int kListWin = 32;                   // segments per staged window, one per lane
-// The list is cut into one chunk of consecutive voxels per warp of the grid. The grid
-// is sized from the capacity (launch_list): the resident CTAs as many times as keeps a
-// chunk within kListChunkMax. The CTAs beyond the
-// resident ones start in order as others end, so the warps at work at any moment
-// write one front of the list (see the figures at k_list).
+// The list is cut into chunks of consecutive voxels: as many per resident warp as keep a
+// chunk within kListChunkMax, from the total that the scan found (never from the caller's
+// capacity). A warp's first chunk goes by its index, further ones by a counter, so the
+// warps at work at any moment write one front of the list (see the figures at k_list).
 constexpr int kListChunkUnit = 128;            // chunks are multiples of a row
 constexpr int kListChunkMin = 256;             // voxels per warp at least
 constexpr int kListChunkMax = 6144;            // and at most
@@ -61,6 +60,8 @@ struct ListParams {
     void *list;              // uint32 or uint64 list, 16-byte aligned
     int64_t capacity;
     int32_t *status;
+    uint32_t *counter;       // chunks taken beyond the warps' first (workspace; zero before
+                             // the launch where the total may take more than one per warp)
 };
 
 // Fixed-point words of a list type: F fraction bits, integer parts on top.
@@ -90,6 +91,15 @@ struct ListFix<uint64_t> {
         return (static_cast<uint64_t>(hi) << 32) | lo;
     }
 };
+
+// Voxels per chunk of a list of V voxels written by n_warps warps.
+__host__ __device__ inline int32_t list_chunk(int64_t V, int64_t n_warps)
+{
+    const int64_t round = n_warps * kListChunkMax;  // voxels of one chunk per warp at most
+    const int64_t chunks = V <= round ? n_warps : n_warps * ((V + round - 1) / round);
+    const int64_t per = ((V + chunks - 1) / chunks + kListChunkUnit - 1) & ~int64_t(kListChunkUnit - 1);
+    return static_cast<int32_t>(per > kListChunkMin ? per : int64_t(kListChunkMin));
+}
 
 // A window of segments as the lanes read it: field by field, so that lanes reading
 // different segments hit different banks.
@@ -141,13 +151,15 @@ __device__ __forceinline__ uint64_t mul_signed(uint32_t k, uint64_t t)
     return static_cast<uint64_t>(static_cast<int64_t>(static_cast<int32_t>(k))) * t;
 }
 
-// One chunk per warp, written front to back. What the chunks' order is worth: with
-// persistent warps taking every n_warps-th chunk the warps drift apart, and 2.07e9
-// 64-bit voxels take 2785 us; with CTAs started in order (or chunks from a global
-// counter) the writes stay one front and take 2308 us (7.2 TB/s). Chunks of 8192 /
-// 12288 voxels at most: 2353 / 2451 us; 2048: 3416 us (the search per chunk). Rows
-// collected in shared memory and stored by 4 KB bulk copies: 2421 us, and 88 instead
-// of 76 us on 64-voxel segments.
+// Chunks in list order, each written front to back by one warp. What the order is worth:
+// with persistent warps taking every n_warps-th chunk the warps drift apart, and 2.07e9
+// 64-bit voxels take 2785 us; with chunks from a counter the writes stay one front and
+// take 2335 us (7.1 TB/s), whatever the list's capacity. (One chunk per warp of a grid sized
+// from the capacity, its CTAs started in order: 2308 us with a capacity of V, but 2552
+// with 3 V and 7016 with 16 V, whose chunks are of 384 voxels.) Chunks of 8192 / 12288
+// voxels at most: 2353 / 2451 us; 2048: 3416 us (the search per chunk). Rows collected in
+// shared memory and stored by 4 KB bulk copies: 2421 us, and 88 instead of 76 us on
+// 64-voxel segments.
 template <typename PackT>
 __global__ void __launch_bounds__(kListThreads, kListCtas) k_list(ListParams p)
 {
@@ -155,7 +167,7 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_list(ListParams p)
     constexpr int kVox = 16 / sizeof(PackT);  // consecutive voxels per lane and row: one 16-byte store
     constexpr int kRow = 32 * kVox;
     __shared__ ListWarpSmem<PackT> s_win[kListWarps];
-    __shared__ int32_t s_go;
+    __shared__ int32_t s_go, s_chunk;
     __shared__ int64_t s_V;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -171,18 +183,18 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_list(ListParams p)
         }
         s_go = go;
         s_V = V;
+        s_chunk = list_chunk(V, static_cast<int64_t>(gridDim.x) * kListWarps);
     }
     __syncthreads();
     if (!s_go) return;
     const int64_t V = s_V;
+    const int32_t chunk = s_chunk;
     PackT *const list = static_cast<PackT *>(p.list);
-    const int64_t n_warps = static_cast<int64_t>(gridDim.x) * kListWarps;
-    const int64_t per = ((V + n_warps - 1) / n_warps + kListChunkUnit - 1) & ~int64_t(kListChunkUnit - 1);
-    const int64_t chunk = max64(kListChunkMin, per);
+    const uint32_t n_warps = gridDim.x * kListWarps;
     const uint32_t le_mask = 0xffffffffu >> (31 - lane);  // this lane and those below
 
-    const int64_t g0 = (static_cast<int64_t>(blockIdx.x) * kListWarps + warp) * chunk;
-    if (g0 < V) {
+    int64_t g0 = static_cast<int64_t>(blockIdx.x * kListWarps + warp) * chunk;
+    while (g0 < V) {
         const int32_t len = static_cast<int32_t>(min64(chunk, V - g0));
         PackT *const out = list + g0;
         int64_t s = warp_find_segment(p.offsets, p.n, g0, lane);
@@ -317,6 +329,10 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_list(ListParams p)
             }
             s += j;
         }
+        if (static_cast<int64_t>(n_warps) * chunk >= V) break;
+        uint32_t next = 0;
+        if (lane == 0) next = atomicAdd(p.counter, 1u);
+        g0 = (static_cast<int64_t>(n_warps) + __shfl_sync(0xffffffffu, next, 0)) * chunk;
     }
 }
 
