@@ -19,17 +19,20 @@
 // The slopes are divided out once per staged segment (a lane per segment of the
 // window), not once per run of voxels.
 //
-// What bounds it: HBM writes for 64-bit lists of long segments, instruction issue
-// for short ones (75 % of issue slots on 64-voxel segments; about 110 instructions a
-// row that holds segment starts, a row being 128 32-bit or 64 64-bit voxels).
-// Measured (GB300, list kernel alone), against runs of 33 voxels per lane stepped by
-// the carry recurrence into a shared stage (long segments) and 32-voxel thread runs
-// with a transposed stage (the rest):
-//   4M log-uniform segments in 4096^3, 64-bit, 2.07e9 voxels   2720 -> 2308 us
-//   1024 segments, 10^9 voxels, 64-bit                         1090 -> 1051 us
-//   1M log-uniform segments in 1000^3, 64-bit, 1.4e8 voxels     301 ->  208 us
-//   300,000 uniform segments in 256^3, 32-bit, 4.2e7 voxels      76 ->   54 us
-//   1M segments of 64 voxels, 32-bit, 6.7e7 voxels               78 ->   76 us
+// What bounds it: HBM writes for 64-bit lists of long segments, instruction issue for
+// short ones (a row is 128 32-bit or 64 64-bit voxels; most of its instructions are three
+// additions and three or four shifts a voxel).
+// Measured (GB300, list kernel alone), against runs of 33 voxels per lane stepped by the
+// carry recurrence into a shared stage (long segments) and 32-voxel thread runs with a
+// transposed stage (the rest); in the middle, rows whose lanes read a segment by eight
+// 4-byte loads, start and step apart, and pack by shifts and masks:
+//   4M log-uniform segments in 4096^3, 64-bit, 2.07e9 voxels   2720 -> 2308 -> 2327 us
+//   1024 segments, 10^9 voxels, 64-bit                         1090 -> 1048 -> 1056 us
+//   1M log-uniform segments in 1000^3, 64-bit, 1.5e8 voxels     301 ->  216 ->  208 us
+//   300,000 uniform segments in 256^3, 32-bit, 4.2e7 voxels      76 ->   52 ->   43 us
+//   1M segments of 64 voxels, 32-bit, 6.7e7 voxels               78 ->   75 ->   63 us
+// (the last: 66 us by 64-voxel thread runs, which a tuning could ask for; the second step of
+// the first two lies in the order of the chunks, see k_list)
 #pragma once
 
 #include <cstdint>
@@ -64,7 +67,8 @@ struct ListParams {
                              // the launch where the total may take more than one per warp)
 };
 
-// Fixed-point words of a list type: F fraction bits, integer parts on top.
+// Fixed-point words of a list type: F fraction bits, integer parts on top. Packing is a
+// chain of funnel shifts, (h << n) | (l >> (32 - n)).
 template <typename PackT>
 struct ListFix;
 
@@ -74,7 +78,7 @@ struct ListFix<uint32_t> {
     // x | y << 10 | z << 20 from the top 10 bits of each word
     static __device__ __forceinline__ uint32_t pack(uint32_t x, uint32_t y, uint32_t z)
     {
-        return (x >> 22) | ((y >> 12) & 0x000ffc00u) | ((z >> 2) & 0x3ff00000u);
+        return __funnelshift_l(x, __funnelshift_l(y, z >> 22, 10), 10);
     }
 };
 
@@ -86,8 +90,8 @@ struct ListFix<uint64_t> {
     {
         const uint32_t xh = static_cast<uint32_t>(x >> 32), yh = static_cast<uint32_t>(y >> 32),
                        zh = static_cast<uint32_t>(z >> 32);
-        const uint32_t lo = (xh >> 11) | ((yh << 10) & 0xffe00000u);
-        const uint32_t hi = (yh >> 22) | ((zh >> 1) & 0x7ffffc00u);
+        const uint32_t lo = __funnelshift_l(xh, yh >> 11, 21);
+        const uint32_t hi = __funnelshift_l(yh, zh >> 11, 10);
         return (static_cast<uint64_t>(hi) << 32) | lo;
     }
 };
@@ -101,13 +105,55 @@ __host__ __device__ inline int32_t list_chunk(int64_t V, int64_t n_warps)
     return static_cast<int32_t>(per > kListChunkMin ? per : int64_t(kListChunkMin));
 }
 
-// A window of segments as the lanes read it: field by field, so that lanes reading
-// different segments hit different banks.
+// A segment of the window: coordinates X = C + p T at position p of the chunk (the
+// segment's X0 less its first position times T, modulo the word), so that a voxel needs
+// neither the segment's start nor its step; and the position where the next one starts.
 template <typename PackT>
-struct ListWarpSmem {
-    PackT X0[3][kListWin];        // coordinates of voxel 0 (fixed point, half added)
-    PackT T[3][kListWin];         // per-voxel steps
-    int32_t rel[kListWin + 1];    // first voxel of each segment, relative to the chunk (+ the next)
+struct ListSeg {
+    PackT C[3], T[3];
+    int32_t next;
+};
+
+// The window as the lanes read it, in words of 16 bytes: two (32-bit) or three loads bring
+// a segment, and lanes that read consecutive segments meet no bank twice.
+template <typename PackT>
+struct ListWarpSmem;
+
+template <>
+struct ListWarpSmem<uint32_t> {
+    uint4 a[kListWin], b[kListWin];
+
+    __device__ __forceinline__ void put(int j, const ListSeg<uint32_t> &g)
+    {
+        a[j] = make_uint4(g.C[0], g.C[1], g.C[2], static_cast<uint32_t>(g.next));
+        b[j] = make_uint4(g.T[0], g.T[1], g.T[2], 0u);
+    }
+    __device__ __forceinline__ ListSeg<uint32_t> get(int j) const
+    {
+        const uint4 u = a[j], v = b[j];
+        return {{u.x, u.y, u.z}, {v.x, v.y, v.z}, static_cast<int32_t>(u.w)};
+    }
+    __device__ __forceinline__ int32_t next(int j) const { return static_cast<int32_t>(a[j].w); }
+};
+
+template <>
+struct ListWarpSmem<uint64_t> {
+    ulonglong2 a[kListWin], b[kListWin], c[kListWin];
+    int32_t nx[kListWin];
+
+    __device__ __forceinline__ void put(int j, const ListSeg<uint64_t> &g)
+    {
+        a[j] = make_ulonglong2(g.C[0], g.C[1]);
+        b[j] = make_ulonglong2(g.C[2], g.T[0]);
+        c[j] = make_ulonglong2(g.T[1], g.T[2]);
+        nx[j] = g.next;
+    }
+    __device__ __forceinline__ ListSeg<uint64_t> get(int j) const
+    {
+        const ulonglong2 u = a[j], v = b[j], w = c[j];
+        return {{u.x, u.y, v.x}, {v.y, w.x, w.y}, nx[j]};
+    }
+    __device__ __forceinline__ int32_t next(int j) const { return nx[j]; }
 };
 
 // Largest s in [0, n) with offsets[s] <= g (offsets[0] <= g < offsets[n]): a
@@ -142,13 +188,6 @@ __device__ __forceinline__ int4 list_quad(const uint64_t (&v)[2])
 {
     return make_int4(static_cast<int>(v[0]), static_cast<int>(v[0] >> 32), static_cast<int>(v[1]),
                      static_cast<int>(v[1] >> 32));
-}
-
-// k t for a signed step count k given in two's complement (modulo the word).
-__device__ __forceinline__ uint32_t mul_signed(uint32_t k, uint32_t t) { return k * t; }
-__device__ __forceinline__ uint64_t mul_signed(uint32_t k, uint64_t t)
-{
-    return static_cast<uint64_t>(static_cast<int64_t>(static_cast<int32_t>(k))) * t;
 }
 
 // Chunks in list order, each written front to back by one warp. What the order is worth:
@@ -191,7 +230,7 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_list(ListParams p)
     const int32_t chunk = s_chunk;
     PackT *const list = static_cast<PackT *>(p.list);
     const uint32_t n_warps = gridDim.x * kListWarps;
-    const uint32_t le_mask = 0xffffffffu >> (31 - lane);  // this lane and those below
+    const uint32_t lt_mask = (1u << lane) - 1u;  // the lanes below
 
     int64_t g0 = static_cast<int64_t>(blockIdx.x * kListWarps + warp) * chunk;
     while (g0 < V) {
@@ -208,18 +247,20 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_list(ListParams p)
                 int32_t r[6];
                 load_record(p.segs, s + lane, r);
                 rel = static_cast<int32_t>(__ldg(p.offsets + s + lane) - g0);
-                sm.rel[lane] = rel;
-                if (lane == wcnt - 1) sm.rel[wcnt] = static_cast<int32_t>(__ldg(p.offsets + s + wcnt) - g0);
                 const uint32_t N = static_cast<uint32_t>(max(abs(r[3] - r[0]), max(abs(r[4] - r[1]), abs(r[5] - r[2]))));
+                ListSeg<PackT> g;
+                g.next = static_cast<int32_t>(__ldg(p.offsets + s + lane + 1) - g0);
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     const int32_t d = r[3 + a] - r[a];
                     const PackT A = static_cast<PackT>(abs(d));
                     const PackT S = A == N ? PackT(1) << Fix::F  // the major axis, and minor ones as long
                                            : ((A << Fix::F) + (N - 1u)) / N;
-                    sm.X0[a][lane] = (static_cast<PackT>(r[a]) << Fix::F) + (PackT(1) << (Fix::F - 1)) - (d < 0 ? 1 : 0);
-                    sm.T[a][lane] = d < 0 ? PackT(0) - S : S;
+                    g.T[a] = d < 0 ? PackT(0) - S : S;
+                    g.C[a] = (static_cast<PackT>(r[a]) << Fix::F) + (PackT(1) << (Fix::F - 1)) - (d < 0 ? 1 : 0) -
+                             static_cast<PackT>(static_cast<typename std::make_signed<PackT>::type>(rel)) * g.T[a];
                 }
+                sm.put(lane, g);
             }
             // the next 32 segments' records and offsets on their way to L1
             if (s + 2 * kListWin <= p.n) {
@@ -227,81 +268,76 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_list(ListParams p)
                 else prefetch_l1(p.offsets + s + kListWin + 4 * (lane - 24));
             }
             __syncwarp();
-            const int32_t wend = sm.rel[wcnt];
+            const int32_t wend = sm.next(wcnt - 1);
+            const int32_t lim = min(wend, len);
             int32_t j = 0;  // the window's segment that holds pos
             while (true) {
                 // a row needs the window to cover it; without that the window moves on
                 // to segment j, or (already there, or the list ends) 32 voxels are taken
-                const bool covered = pos + kRow <= min(wend, len);
+                const bool covered = pos + kRow <= lim;
                 if (!covered && j > 0 && wend < len) break;
-                // the segments that start in the row after its first voxel, by the first
-                // lane whose voxels all follow the start; two of them at one lane: short
-                // segments, 32 voxels at a time
+                // the segments that start in the row after its first voxel (or right after
+                // the row), by the lane that holds the voxel before the start; two of them
+                // at one lane: short segments, 32 voxels at a time
                 const int32_t b = rel - pos;
-                const bool inside = b > 0 && b < kRow;
-                const uint32_t starts = __reduce_or_sync(0xffffffffu, inside ? 2u << ((b - 1) / kVox) : 0u);
-                if (covered && starts == 0u) {
-                    const int32_t e = sm.rel[j + 1];
-                    if (e - pos >= kRow) {
-                        // rows inside one segment
-                        const uint32_t k = static_cast<uint32_t>(pos + kVox * lane - sm.rel[j]);
-                        const PackT tx = sm.T[0][j], ty = sm.T[1][j], tz = sm.T[2][j];
-                        PackT x = sm.X0[0][j] + k * tx, y = sm.X0[1][j] + k * ty, z = sm.X0[2][j] + k * tz;
-                        const int32_t stop = min(e, len) - kRow;
-                        int4 *o = reinterpret_cast<int4 *>(out + pos) + lane;
+                const bool inside = b > 0 && b <= kRow;
+                const uint32_t starts = __reduce_or_sync(0xffffffffu, inside ? 1u << ((b - 1) / kVox) : 0u);
+                if (covered && starts == 0u) {  // rows inside one segment
+                    const ListSeg<PackT> g = sm.get(j);
+                    const PackT p0 = static_cast<PackT>(pos + kVox * lane);
+                    PackT x = g.C[0] + p0 * g.T[0], y = g.C[1] + p0 * g.T[1], z = g.C[2] + p0 * g.T[2];
+                    const int32_t stop = min(g.next, len) - kRow;
+                    int4 *o = reinterpret_cast<int4 *>(out + pos) + lane;
 #pragma unroll 2
-                        for (; pos <= stop; pos += kRow) {
-                            PackT v[kVox];
+                    for (; pos <= stop; pos += kRow) {
+                        PackT v[kVox];
 #pragma unroll
-                            for (int i = 0; i < kVox; ++i) {
-                                v[i] = Fix::pack(x, y, z);
-                                const uint32_t f = i + 1 < kVox ? 1u : static_cast<uint32_t>(kRow - kVox + 1);
-                                x += f * tx;
-                                y += f * ty;
-                                z += f * tz;
-                            }
-                            *o = list_quad(v);
-                            o += 32;
+                        for (int i = 0; i < kVox; ++i) {
+                            v[i] = Fix::pack(x, y, z);
+                            const uint32_t f = i + 1 < kVox ? 1u : static_cast<uint32_t>(kRow - kVox + 1);
+                            x += f * g.T[0];
+                            y += f * g.T[1];
+                            z += f * g.T[2];
                         }
-                        if (pos >= len) break;
-                        if (e <= pos) {
-                            ++j;
-                            if (j >= wcnt) break;
-                        }
-                        continue;
+                        *o = list_quad(v);
+                        o += 32;
                     }
+                    if (pos >= len) break;
+                    if (g.next <= pos) {
+                        ++j;
+                        if (j >= wcnt) break;
+                    }
+                    continue;
                 }
-                // (a start among the last lane's voxels has no such lane)
                 const int32_t n_in = __popc(__ballot_sync(0xffffffffu, inside));
-                const int32_t n_last = __popc(__ballot_sync(0xffffffffu, inside && b > kRow - kVox));
-                if (covered && n_last <= 1 && __popc(starts) + n_last == n_in) {
+                if (covered && __popc(starts) == n_in) {
                     // a row with segment starts, at most one per lane
                     const int32_t p0 = pos + kVox * lane;
-                    const int32_t jl = j + __popc(starts & le_mask);
-                    const int32_t c = sm.rel[jl + 1] - p0;  // this lane's voxels from c on are the next segment's
-                    const uint32_t k = static_cast<uint32_t>(p0 - sm.rel[jl]);
-                    const PackT tx = sm.T[0][jl], ty = sm.T[1][jl], tz = sm.T[2][jl];
-                    PackT x = sm.X0[0][jl] + k * tx, y = sm.X0[1][jl] + k * ty, z = sm.X0[2][jl] + k * tz;
+                    const int32_t jl = j + __popc(starts & lt_mask);
+                    const ListSeg<PackT> g = sm.get(jl);
+                    PackT x = g.C[0] + static_cast<PackT>(p0) * g.T[0], y = g.C[1] + static_cast<PackT>(p0) * g.T[1],
+                          z = g.C[2] + static_cast<PackT>(p0) * g.T[2];
                     PackT v[kVox];
 #pragma unroll
                     for (int i = 0; i < kVox; ++i) {
                         v[i] = Fix::pack(x, y, z);
-                        x += tx;
-                        y += ty;
-                        z += tz;
+                        x += g.T[0];
+                        y += g.T[1];
+                        z += g.T[2];
                     }
+                    const int32_t c = g.next - p0;  // this lane's voxels from c on are the next segment's
                     if (c < kVox) {
-                        const uint32_t back = 0u - static_cast<uint32_t>(c - 1);  // voxel 1 is its step 1 - c
-                        const PackT ux = sm.T[0][jl + 1], uy = sm.T[1][jl + 1], uz = sm.T[2][jl + 1];
-                        x = sm.X0[0][jl + 1] + mul_signed(back, ux);
-                        y = sm.X0[1][jl + 1] + mul_signed(back, uy);
-                        z = sm.X0[2][jl + 1] + mul_signed(back, uz);
+                        const ListSeg<PackT> h = sm.get(jl + 1);
+                        const PackT p1 = static_cast<PackT>(p0 + 1);
+                        x = h.C[0] + p1 * h.T[0];
+                        y = h.C[1] + p1 * h.T[1];
+                        z = h.C[2] + p1 * h.T[2];
 #pragma unroll
                         for (int i = 1; i < kVox; ++i) {
                             if (i >= c) v[i] = Fix::pack(x, y, z);
-                            x += ux;
-                            y += uy;
-                            z += uz;
+                            x += h.T[0];
+                            y += h.T[1];
+                            z += h.T[2];
                         }
                     }
                     reinterpret_cast<int4 *>(out + pos)[lane] = list_quad(v);
@@ -310,21 +346,19 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_list(ListParams p)
                 } else {
                     // 32 voxels, one per lane (the window covers them: 32 segments hold at
                     // least 32 voxels): a bit for each start, and each lane counts the bits
-                    // up to its own position
+                    // before its own position
                     if (wend < len && pos + 32 > wend) break;
-                    const uint32_t bits = __reduce_or_sync(0xffffffffu, (b > 0 && b < 32) ? 1u << b : 0u);
-                    const int32_t jl = j + __popc(bits & le_mask);
-                    const uint32_t k = static_cast<uint32_t>(pos + lane - sm.rel[jl]);
-                    const PackT x = sm.X0[0][jl] + k * sm.T[0][jl], y = sm.X0[1][jl] + k * sm.T[1][jl],
-                                z = sm.X0[2][jl] + k * sm.T[2][jl];
-                    if (pos + lane < len) out[pos + lane] = Fix::pack(x, y, z);
+                    const uint32_t bits = __reduce_or_sync(0xffffffffu, (b > 0 && b <= 32) ? 1u << (b - 1) : 0u);
+                    const ListSeg<PackT> g = sm.get(j + __popc(bits & lt_mask));
+                    const PackT p0 = static_cast<PackT>(pos + lane);
+                    if (pos + lane < len)
+                        out[pos + lane] = Fix::pack(g.C[0] + p0 * g.T[0], g.C[1] + p0 * g.T[1], g.C[2] + p0 * g.T[2]);
                     pos += 32;
                     j += __popc(bits);
                 }
-                if (pos >= len) break;
-                if (sm.rel[j + 1] <= pos) {  // the next row starts a segment
-                    ++j;
-                    if (j >= wcnt) break;
+                if (pos >= lim) {  // the list's end, or the window's
+                    j = wcnt;
+                    break;
                 }
             }
             s += j;
