@@ -274,15 +274,16 @@ bool uses_bricks(int64_t n, vox_dims dims, size_t ws_bytes, BrickGeom *G, size_t
 
 int grid_ctas(const void *kernel, int threads, size_t smem);
 
-// The binning passes: persistent grids (SMs x CTAs per SM, no more CTAs than
-// the segments fill), warps taking batches of segments.
+// The binning passes: persistent grids (SMs x CTAs per SM, no more CTAs than the
+// segments, or the lanes' other tasks, fill), warps taking batches of segments.
 template <int kPer>
-vox_status launch_bin_grid(void (*k)(BinParams), const BinParams &bp, int64_t n, cudaStream_t stream)
+vox_status launch_bin_grid(void (*k)(BinParams), const BinParams &bp, int64_t n, cudaStream_t stream, int64_t tasks = 0)
 {
     int grid = grid_ctas(reinterpret_cast<const void *>(k), kBinThreads, 0);
     if (grid <= 0) return VOX_ERR_CUDA;
     constexpr int kCta = kBinWarps * 32 * kPer;  // segments of a CTA's first batches
-    grid = static_cast<int>(std::min<int64_t>(grid, (n + kCta - 1) / kCta));
+    grid = static_cast<int>(
+        std::min<int64_t>(grid, std::max((n + kCta - 1) / kCta, (tasks + kBinThreads - 1) / kBinThreads)));
     k<<<static_cast<unsigned>(grid), kBinThreads, 0, stream>>>(bp);
     return cudaGetLastError() == cudaSuccess ? VOX_OK : VOX_ERR_CUDA;
 }
@@ -292,7 +293,10 @@ vox_status launch_bin_grid(void (*k)(BinParams), const BinParams &bp, int64_t n,
 template <bool kEuclid, bool kBatched>
 vox_status launch_bin_t(const BinParams &bp, bool scatter, int64_t n, cudaStream_t stream)
 {
-    if (scatter) return launch_bin_grid<2>(k_bin_scatter<kEuclid, kBatched, 2>, bp, n, stream);
+    if (scatter) {  // which also looks for hot bricks
+        const int64_t tasks = bp.G.n_bricks << clear_split(bp.fresh != 0, bp.G.n_bricks);
+        return launch_bin_grid<2>(k_bin_scatter<kEuclid, kBatched, 2>, bp, n, stream, tasks);
+    }
     return n > (int64_t(1) << 20) ? launch_bin_grid<4>(k_bin_count<kEuclid, kBatched, 4>, bp, n, stream)
                                   : launch_bin_grid<2>(k_bin_count<kEuclid, kBatched, 2>, bp, n, stream);
 }

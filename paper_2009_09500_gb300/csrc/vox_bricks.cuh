@@ -632,28 +632,35 @@ __device__ __forceinline__ void clear_brick(const BrickGeom &G, int64_t lb, uint
     }
 }
 
+// A hot brick of a fresh volume is cleared by 2^clear_split warps (one clears 64 KB in 20
+// to 150 us).
+__host__ __device__ inline int32_t clear_split(bool fresh, int64_t n_bricks) { return fresh && n_bricks <= 4096 ? 5 : 0; }
+
 // The bricks to be walked in parts: their parts listed, their words of a fresh volume
-// cleared, each brick by `split` warps (one clears 64 KB in 20 to 150 us). Task
-// i = (brick, c of split) goes to warp i mod (warps of the grid), a lane each.
+// cleared. Task i = (brick, part of the clearing) goes to warp i mod (warps of the grid),
+// a lane each; the grid has a lane for every task as far as the CTAs are resident
+// (launch_bin_t), since a round costs two dependent loads: 500 segments in a fresh 1024^3
+// volume (1,024 bricks) took 183 us a call by the one CTA that their number fills, 130 so.
 template <bool kBatched>
 __device__ __forceinline__ void find_hot(const BinParams &p)
 {
     const int lane = threadIdx.x & 31;
     const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    const int64_t limit = hot_pieces(__ldg(p.brick_off + p.G.n_slots));
+    const int64_t total = __ldg(p.brick_off + p.G.n_slots), limit = hot_pieces(total);
+    if (total <= limit) return;  // no brick has more
     const int64_t slots = static_cast<int64_t>(kPieceClasses) * p.G.reps;
-    const int32_t split = p.fresh && p.G.n_bricks <= 4096 ? 32 : 1;
-    const int64_t tasks = p.G.n_bricks * split;
+    const int32_t log_split = clear_split(p.fresh != 0, p.G.n_bricks), split = 1 << log_split;
+    const int64_t tasks = p.G.n_bricks << log_split;
     for (int64_t i0 = gw; i0 < tasks; i0 += 32 * nw) {
-        const int64_t i = i0 + lane * nw, b = i / split;
+        const int64_t i = i0 + lane * nw, b = i >> log_split;
         int64_t lo = 0, hi = 0;
         if (i < tasks) {
             lo = __ldg(p.brick_off + b * slots);
             hi = __ldg(p.brick_off + (b + 1) * slots);
         }
         uint32_t hot = __ballot_sync(0xffffffffu, hi - lo > limit);
-        if (hi - lo > limit && i % split == 0) {
+        if (hi - lo > limit && (i & (split - 1)) == 0) {
             const int32_t parts = static_cast<int32_t>((hi - lo + limit - 1) / limit);
             const int64_t per = ((hi - lo + parts - 1) / parts + 31) & ~int64_t(31);
             const uint32_t at = atomicAdd(p.n_hot, static_cast<uint32_t>(parts));
@@ -661,8 +668,8 @@ __device__ __forceinline__ void find_hot(const BinParams &p)
                 p.hot[at + e] = HotPart{b, min64(lo + e * per, hi), min64(lo + (e + 1) * per, hi)};
         }
         while (p.fresh && hot) {
-            const int64_t t = i0 + (__ffs(hot) - 1) * nw, hb = t / split;
-            const int32_t c = static_cast<int32_t>(t % split);
+            const int64_t t = i0 + (__ffs(hot) - 1) * nw, hb = t >> log_split;
+            const int32_t c = static_cast<int32_t>(t & (split - 1));
             hot &= hot - 1;
             if constexpr (kBatched) {
                 const int32_t k = __ldg(p.brick_scene + hb);
