@@ -148,13 +148,12 @@ __device__ __forceinline__ int32_t piece_class_desc(int32_t len)
     return kPieceClasses - 1 - cls;
 }
 
-// Slots fit 31 bits: with replicas there are at most 32768 bricks, else at
-// most 2^26 bricks and one replica.
-__device__ __forceinline__ uint32_t piece_slot(const BrickGeom &G, int32_t brick, int32_t len, int32_t rep)
+// The first slot of a piece of the brick (the replica is added to it). Slots fit 31 bits:
+// with replicas there are at most 32768 bricks, else at most 2^26 bricks and one replica.
+__device__ __forceinline__ uint32_t piece_slot(int32_t reps, int32_t brick, int32_t len)
 {
     return (static_cast<uint32_t>(brick) * kPieceClasses + static_cast<uint32_t>(piece_class_desc(len))) *
-               static_cast<uint32_t>(G.reps) +
-           static_cast<uint32_t>(rep);
+           static_cast<uint32_t>(reps);
 }
 
 // A segment as the brick kernel enters it, one 32-byte sector, written once by the
@@ -325,9 +324,9 @@ struct PieceWalker {
 constexpr int32_t kPieceMaxLen = 64;
 
 // piece = segment (32 bits) | first step (22 bits) | length - 1 (10 bits)
-__device__ __forceinline__ uint64_t pack_piece(int64_t seg, int32_t k_lo, int32_t len)
+__device__ __forceinline__ uint64_t pack_piece(uint32_t seg, int32_t k_lo, int32_t len)
 {
-    return static_cast<uint64_t>(static_cast<uint32_t>(seg)) | (static_cast<uint64_t>(k_lo) << 32) |
+    return static_cast<uint64_t>(seg) | (static_cast<uint64_t>(k_lo) << 32) |
            (static_cast<uint64_t>(len - 1) << 54);
 }
 
@@ -471,7 +470,8 @@ __device__ __forceinline__ void bin_unit(const BinParams &p, const BinWarpSmem<k
     int64_t slot_base;
     const BrickGeom *Gp = segment_geom<kBatched>(p, s, slot_base);
     const bool few = Gp->n_bricks <= kFewBricks;
-    const int32_t rep = static_cast<int32_t>(few ? s >> 5 : s) & (Gp->reps - 1);
+    const int32_t reps = Gp->reps;
+    const int64_t base = slot_base + (static_cast<int32_t>(few ? s >> 5 : s) & (reps - 1));
     int32_t r[6];
 #pragma unroll
     for (int a = 0; a < 6; ++a) r[a] = sm.rec[a][j];
@@ -484,7 +484,7 @@ __device__ __forceinline__ void bin_unit(const BinParams &p, const BinWarpSmem<k
             more = pw.next(b, k_lo, len);
         }
         const int32_t part = min(len, kPieceMaxLen);
-        emit(slot_base + piece_slot(*Gp, b, part, rep), s, k_lo, part, few);
+        emit(base + piece_slot(reps, b, part), static_cast<uint32_t>(s), k_lo, part, few);
         k_lo += part;
         len -= part;
     }
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(kBinThreads, kBinCtas) k_bin_count(BinParams p
     // a batch reads the scene map and numbering, valid only without an error
     // (decided by the whole warp: the walk's shuffles and votes need every lane)
     if (kBatched && __any_sync(0xffffffffu, ld_volatile_i32(p.status) != 0)) return;
-    bin_loop<kEuclid, kBatched, false, kPer>(p, [&](int64_t slot, int64_t, int32_t, int32_t, bool few) {
+    bin_loop<kEuclid, kBatched, false, kPer>(p, [&](int64_t slot, uint32_t, int32_t, int32_t, bool few) {
         if (few) {
             const SlotGroup g(slot);
             if (g.rank == 0) atomicAdd(p.brick_count + slot, __popc(g.lanes));
@@ -685,8 +685,10 @@ __device__ __forceinline__ void find_hot(const BinParams &p)
 // Pieces written into their slots (persistent grid), and the slope table. p.G.n_slots: the number of
 // slots (all scenes' when batched). Bound by the latency of the returning atomics:
 // slot reservations of two pieces of a lane are in flight together before their
-// stores (4M log-uniform segments: 1075 us; four, or one held while the walk goes on:
-// 9 to 10 % more).
+// stores (4M log-uniform segments: 1075 us; one: 1136; four, or one held while the walk
+// goes on: 9 to 10 % more). The first of the two waits in shared memory: in registers the
+// batched instance spills (serve-sized batches of five scenes 219 -> 206 us, 48 uneven
+// scenes 103 -> 98).
 template <bool kEuclid, bool kBatched, int kPer>
 __global__ void __launch_bounds__(kBinThreads, kBinCtas) k_bin_scatter(BinParams p)
 {
@@ -695,40 +697,32 @@ __global__ void __launch_bounds__(kBinThreads, kBinCtas) k_bin_scatter(BinParams
     if (__any_sync(0xffffffffu, ld_volatile_i32(p.status) != 0)) return;
     if (__ldg(p.brick_off + p.G.n_slots) > p.capacity) return;  // the volume falls back to atomics
     find_hot<kBatched>(p);
-    constexpr int kBatch = 2;
-    int64_t bb[kBatch];
-    uint64_t val[kBatch];
-    int nb = 0;
-    auto flush = [&]() {
-        unsigned long long pos[kBatch];
-#pragma unroll
-        for (int e = 0; e < kBatch; ++e)
-            if (e < nb) pos[e] = atomicAdd(reinterpret_cast<unsigned long long *>(p.cursor + bb[e]), 1ull);
-#pragma unroll
-        for (int e = 0; e < kBatch; ++e)
-            if (e < nb) p.pieces[pos[e]] = val[e];
-        nb = 0;
+    __shared__ ulonglong2 s_pending[kBinThreads];  // a slot and its piece per thread
+    bool pending = false;
+    auto reserve = [&](uint64_t slot, uint64_t pieces) {
+        return atomicAdd(reinterpret_cast<unsigned long long *>(p.cursor + slot), static_cast<unsigned long long>(pieces));
     };
-    bin_loop<kEuclid, kBatched, true, kPer>(p, [&](int64_t slot, int64_t seg, int32_t k, int32_t len, bool few) {
+    bin_loop<kEuclid, kBatched, true, kPer>(p, [&](int64_t slot, uint32_t seg, int32_t k, int32_t len, bool few) {
         if (few) {
             const SlotGroup g(slot);
             unsigned long long at = 0;
-            if (g.rank == 0)
-                at = atomicAdd(reinterpret_cast<unsigned long long *>(p.cursor + slot),
-                               static_cast<unsigned long long>(__popc(g.lanes)));
+            if (g.rank == 0) at = reserve(slot, __popc(g.lanes));
             at = __shfl_sync(g.lanes, at, g.leader);
             p.pieces[at + g.rank] = pack_piece(seg, k, len);
             return;
         }
-#pragma unroll
-        for (int e = 0; e < kBatch; ++e)
-            if (e == nb) {
-                bb[e] = slot;
-                val[e] = pack_piece(seg, k, len);
-            }
-        if (++nb == kBatch) flush();
+        const uint64_t piece = pack_piece(seg, k, len);
+        if (pending) {
+            const ulonglong2 first = s_pending[threadIdx.x];
+            const unsigned long long at0 = reserve(first.x, 1), at1 = reserve(slot, 1);
+            p.pieces[at0] = first.y;
+            p.pieces[at1] = piece;
+        } else {
+            s_pending[threadIdx.x] = make_ulonglong2(static_cast<uint64_t>(slot), piece);
+        }
+        pending = !pending;
     });
-    if (nb) flush();
+    if (pending) p.pieces[reserve(s_pending[threadIdx.x].x, 1)] = s_pending[threadIdx.x].y;
 }
 
 struct BrickParams {
@@ -816,8 +810,8 @@ __device__ __forceinline__ void merge_brick(const uint32_t *bits, const BrickGeo
         // 16-byte units (a brick row holds bxw / 4 of them): the brick's first word
         // in a row, X0 / 32, is a multiple of bxw and the volume's rows are whole
         // 16-byte units, so every unit is aligned and lies in or beyond the row
-        // as a whole; four units per thread in flight
-        constexpr int kGroup4 = 4;
+        // as a whole; three units per thread in flight (four spill)
+        constexpr int kGroup4 = 3;
         const uint4 *b4 = reinterpret_cast<const uint4 *>(bits);
         uint4 *m4 = reinterpret_cast<uint4 *>(mask);
         const int32_t units = G.words >> 2;
@@ -934,7 +928,11 @@ __device__ __forceinline__ void take_brick(const BrickParams &p, bool overflow, 
     int64_t first_slot;
     if constexpr (kBatched) {  // the brick's scene and its geometry
         const int32_t k = __ldg(p.brick_scene + b);
-        I.geom = p.sb[k].G;
+        // word by word: the thread's walk waits with its state in registers
+        const int32_t *from = reinterpret_cast<const int32_t *>(&p.sb[k].G);
+        int32_t *to = reinterpret_cast<int32_t *>(&I.geom);
+#pragma unroll 1
+        for (int i = 0; i < static_cast<int>(sizeof(BrickGeom) / 4); ++i) to[i] = from[i];
         I.bmask = p.sb[k].mask;
         lb = b - p.sb[k].brick_base;
         first_slot = p.sb[k].slot_base + lb * kPieceClasses * I.geom.reps;
@@ -974,9 +972,11 @@ __device__ __forceinline__ void take_brick(const BrickParams &p, bool overflow, 
 // volume, each z quarter by a copy of its own, so that the next brick clears a
 // quarter while the others are still being read.
 // Bound by the shared memory's atomics (32 random words take 3.5 wavefronts of two
-// cycles: 4.8 voxels per cycle and SM, 1.37 ms of the 4M-segment batch's 2.72 ms), and
+// cycles: 4.8 voxels per cycle and SM, 1.37 ms of the 4M-segment batch's 2.68 ms), and
 // by the CTA's wait for its longest group and for its own store between bricks. The
-// walk must not spill: 24 bytes at 64 registers cost 2.89 -> 3.29 ms (59 are used).
+// walk must not spill: 24 bytes at 64 registers cost 2.89 -> 3.29 ms. No instance does
+// (the batched one spilled 28 bytes, most of them where bricks are merged and tickets
+// taken: 48 uneven scenes 243 -> 231 us without, five served scenes 378 -> 369).
 template <bool kEuclid, bool kBatched, bool kWide>
 __global__ void __launch_bounds__(kBrickThreads) k_brick_volume(const __grid_constant__ BrickParams p,
                                                                 const __grid_constant__ CUtensorMap tmap)
@@ -992,12 +992,12 @@ __global__ void __launch_bounds__(kBrickThreads) k_brick_volume(const __grid_con
     // pieces that did not fit: the gated atomics pass ORs the voxels in (after a
     // fresh volume has been cleared here, brick by brick)
     const bool overflow = __ldg(p.brick_off + p.G.n_slots) > p.capacity;
-    if (overflow && p.bricked) {  // no atomics fallback for this layout
+    if (!kBatched && overflow && p.bricked) {  // no atomics fallback for this layout
         if (blockIdx.x == 0 && t == 0) set_status(p.status, kStPieces);
         return;
     }
     if (overflow && !p.fresh) return;
-    const bool async_store = p.use_tma || p.bricked;  // the bitmap leaves by the bulk-copy unit
+    const bool async_store = !kBatched && (p.use_tma || p.bricked);  // the bitmap leaves by the bulk-copy unit
     const int64_t total_bricks = p.G.n_bricks;
     using St = typename std::conditional<kEuclid, EuclidStepper<uint32_t, uint32_t>, Stepper<uint32_t, uint32_t>>::type;
     // a piece's slope table entry (in a wide volume the piece's segment is entered by division)
