@@ -58,10 +58,23 @@ class ServeRequest:
         return self.n * (2 + max(self.dims) // 32) + 1024
 
     @property
+    def bricks(self) -> int:
+        """Bricks of the volume (the shape that include/vox.h documents for rows of whole
+        words); 0 when its width is no multiple of 32."""
+        w, h, d = self.dims
+        if w % 32:
+            return 0
+        b0 = min(256, 1 << (w.bit_length() - 1))
+        b1, b2 = {32: (256, 128), 64: (128, 128), 128: (128, 64), 256: (64, 64)}[b0]
+        return -(-w // b0) * -(-h // b1) * -(-d // b2)
+
+    @property
     def device_bytes(self) -> int:
-        """Volume + segments + workspace share (scan, 32-byte slopes and brick pieces)
-        of this request."""
-        return self.mask_bytes + 24 * self.n + (16 + 32) * self.n + 8 * self.piece_capacity + 256
+        """Volume + segments + workspace share of this request: scan, scene map, 32-byte
+        slopes, brick pieces, the slot counters of its bricks (20 bytes for each of 13
+        length classes and at most 32 replicas) and what a batch has once."""
+        return (self.mask_bytes + 24 * self.n + (16 + 32) * self.n + 8 * self.piece_capacity
+                + 13 * 32 * 21 * self.bricks + (1 << 15))
 
     @property
     def latency_ms(self) -> float:
