@@ -7,11 +7,15 @@ and caches it in a JSON file keyed by the GPU name and a workload class, so a
 later run with a similar workload reuses it without measuring.
 
 Tuned knobs (see include/vox.h, vox_tuning):
-  run_len      voxels per thread run in the atomic volume kernel (16, 32 or 64)
+  run_len      voxels per thread run in the atomic volume kernel (16, 32 or 64); no
+               effect on a list alone or on a volume by bricks
   volume_path  bricks when the workspace allows (auto), per-voxel atomics, or
                per-voxel atomics merged across the warp
   ctas_per_sm  persistent CTAs per SM (0 = occupancy maximum, or fewer)
-  list_runs    no effect any more (a list alone has one kernel)
+  list_runs    no effect (a list alone has one kernel)
+
+Candidates that differ only in knobs without effect on the workload launch the same
+work, and one of them is timed.
 """
 
 from __future__ import annotations
@@ -29,6 +33,24 @@ CANDIDATES = [
     for c in (0, 2)
 ] + [{"run_len": r, "volume_path": vox.VOLUME_AUTO, "ctas_per_sm": 0, "list_runs": 1} for r in (32, 64)] + [
     {"run_len": 32, "volume_path": vox.VOLUME_AUTO, "ctas_per_sm": c, "list_runs": 2} for c in (0, 4)]
+
+
+def effective(params: dict, dims=None, flags: int | None = None) -> tuple:
+    """The knobs of a tuning that reach a kernel on a workload (its volume's dims and
+    output flags, as far as they are known): tunings that agree in them launch the same
+    work. A volume by bricks takes no run length; where the workspace lets it fall back
+    to atomics it launches what VOLUME_ATOMIC does, a candidate of its own."""
+    run_len = params.get("run_len", 0) or 32
+    path = params.get("volume_path", 0)
+    if flags is not None:
+        if not flags & vox.OUT_BITMASK:
+            run_len = path = 0
+        elif path == vox.VOLUME_AUTO and dims is not None:
+            if int(dims[0]) % 32 == 0:
+                run_len = 0
+            else:
+                path = vox.VOLUME_ATOMIC
+    return run_len, path, params.get("ctas_per_sm", 0)
 
 
 def default_cache_path() -> str:
@@ -86,13 +108,19 @@ def measure(run, reps: int = 5, flush_bytes: int = 256 << 20) -> float:
     return sum(ts) / len(ts)
 
 
-def tune(run, candidates=None, reps: int = 5) -> tuple[dict, dict]:
-    """Time `run` under every candidate tuning; returns (best, {name: ms}).
-    The tuning in force on return is the best one."""
+def tune(run, candidates=None, reps: int = 5, dims=None, flags: int | None = None) -> tuple[dict, dict]:
+    """Time `run` under every candidate tuning that launches other work than the ones
+    before it (for a workload of these dims and flags, where given); returns (best,
+    {name: ms}). The tuning in force on return is the best one."""
     candidates = candidates or CANDIDATES
     timings = {}
+    seen = set()
     best, best_ms = None, float("inf")
     for c in candidates:
+        launches = effective(c, dims, flags)
+        if launches in seen:
+            continue
+        seen.add(launches)
         apply(c)
         ms = measure(run, reps)
         timings[json.dumps(c, sort_keys=True)] = ms
@@ -113,7 +141,7 @@ def get_or_tune(run, n_segments: int, total_voxels: int, dims, flags: int, cache
         params = cache[key]["params"]
         apply(params)
         return {"params": params, "key": key, "cached": True}
-    best, timings = tune(run, reps=reps)
+    best, timings = tune(run, reps=reps, dims=dims, flags=flags)
     cache[key] = {"params": best, "timings_ms": timings}
     save_cache(cache, cache_path)
     return {"params": best, "key": key, "cached": False, "timings_ms": timings}
