@@ -88,23 +88,27 @@ def _kernel_source_hash() -> str:
 
 def _recorded_field(workload_key: str, kernels, field):
     """Sum of `field` over `kernels` of one workload in the committed ncu record,
-    if every entry was taken on the current kernel sources with the launch
-    tuning now in force (else None)."""
+    if every entry was taken on the current kernel sources with a launch tuning
+    that launches the same work as the one now in force (else None). The recorded
+    workloads' widths are multiples of 32."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
     try:
         with open(path) as f:
             rec = json.load(f)
     except (OSError, ValueError):
         return None
-    from paper_2009_09500_gb300 import vox
+    from paper_2009_09500_gb300 import autotune, vox
 
-    now = vox.vox_get_tuning()
+    def launches(tuning):
+        return autotune.effective(tuning, (32, 32, 32), vox.OUT_LIST32 | vox.OUT_BITMASK)
+
+    now = launches(vox.vox_get_tuning())
     total = 0.0
     for k in kernels:
         ent = rec.get(f"{workload_key}/{k}")
         if not ent or ent.get("source_hash") != _kernel_source_hash() or field not in ent:
             return None
-        if ent.get("tuning") is not None and ent["tuning"] != now:
+        if ent.get("tuning") is not None and launches(ent["tuning"]) != now:
             return None
         total += float(ent[field])
     return total
