@@ -288,8 +288,8 @@ vox_status launch_bin_grid(void (*k)(BinParams), const BinParams &bp, int64_t n,
     return cudaGetLastError() == cudaSuccess ? VOX_OK : VOX_ERR_CUDA;
 }
 
-// Segments per lane and batch (the figures at bin_loop): two to scatter, and to count
-// until four leave every warp of the grid about two batches.
+// Segments per lane and batch: two to scatter, and to count up to 2^20 segments, about where
+// four become the better (the figures at bin_loop).
 template <bool kEuclid, bool kBatched>
 vox_status launch_bin_t(const BinParams &bp, bool scatter, int64_t n, cudaStream_t stream)
 {

@@ -430,11 +430,15 @@ __device__ __forceinline__ void load_record(const int32_t *segs, int64_t s, int3
 //   200,000 uniform segments, 512^3                  35 +   50 ->  22 +   30
 //   1,000 uniform segments, 512 x 300 x 200          13 +   33 ->   7 +   13
 // kPer segments per lane and batch: more of them fill the rounds of equal octaves
-// better, fewer keep more warps busy. Counting + scattering with four and two: 48 uneven
-// scenes 59 + 110 and 65 + 100; 5 scenes of 1.3 M segments 161 + 241 and 157 + 203; 1M
-// segments of 64 voxels 27 + 51 and 24 + 49, 3M 67 + 147 and 68 + 138; log-uniform 260,000
-// 14 + 31 and 14 + 26, 1M 80 + 177 and 83 + 187, 3M 326 + 859 and 347 + 839 (4M with one:
-// 653 + 1191). launch_bin_t takes two, and four to count more than 2^20 segments.
+// better, fewer keep more warps busy. launch_bin_t scatters with two at any size (with
+// four: 48 uneven scenes 110 against 100 us, 5 scenes of 1.3 M segments 241 against 203, 1M
+// 64-voxel segments 51 against 49, log-uniform 3M 859 against 839; 4M with one 1191). It
+// counts with two up to 2^20 segments and with four beyond (two against four, us):
+//   log-uniform, 2048^3   0.7M 60 : 67,  1.1M 91 : 92,  1.3M 105 : 98,  2.5M 195 : 178,  5M 383 : 340
+//   64 voxels, 1024^3     0.7M 22 : 25,  1.1M 30 : 33,  1.3M  30 : 31,  2.5M  54 :  55,  5M 108 : 107
+//   uniform, 512^3        0.7M 64 : 68,  1.1M 86 : 85,  1.3M 147 : 153, 2.5M 210 : 209,  5M 503 : 504
+//   five served scenes    1.3M 203 : 202, 1.7M 148 : 144, 296 : 270 and 337 : 326, 2.2M 265 : 239
+//   60, 70, 90, 110, 256 uneven scenes  60 : 64, 88 : 76, 87 : 91, 123 : 116, 240 : 231
 // A lane per piece, its step and brick found by fixed-point slopes, takes about 300
 // instructions a piece (779 + 1128 us on the first).
 constexpr int kBinThreads = 256;
