@@ -402,13 +402,6 @@ __device__ __forceinline__ const BrickGeom *segment_geom(const BinParams &p, int
     }
 }
 
-__device__ __forceinline__ void load_record(const int32_t *segs, int64_t s, int32_t *r)
-{
-    const int2 *p = reinterpret_cast<const int2 *>(segs + 6 * s);
-    const int2 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);
-    r[0] = a.x; r[1] = a.y; r[2] = b.x; r[3] = b.y; r[4] = c.x; r[5] = c.y;
-}
-
 // Binning work loop, shared by the counting and the scattering pass (CTAs of
 // kBinThreads threads, persistent grid). A warp takes batches of 32 kPer consecutive
 // segments and cuts their steps into units of kBinUnit, the last one of a segment

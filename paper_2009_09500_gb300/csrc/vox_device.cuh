@@ -46,6 +46,14 @@ __device__ __forceinline__ int32_t ld_volatile_i32(const int32_t *p)
     return *reinterpret_cast<const volatile int32_t *>(p);
 }
 
+// Segment s as (x0, y0, z0, x1, y1, z1); segs 8-byte aligned.
+__device__ __forceinline__ void load_record(const int32_t *segs, int64_t s, int32_t *r)
+{
+    const int2 *p = reinterpret_cast<const int2 *>(segs + 6 * s);
+    const int2 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);
+    r[0] = a.x; r[1] = a.y; r[2] = b.x; r[3] = b.y; r[4] = c.x; r[5] = c.y;
+}
+
 __device__ __forceinline__ uint32_t smem_addr(const void *p)
 {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));

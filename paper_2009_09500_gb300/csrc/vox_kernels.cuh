@@ -23,6 +23,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "vox_bricks.cuh"
 #include "vox_device.cuh"
 
 namespace vox {
