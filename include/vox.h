@@ -166,9 +166,8 @@ vox_status vox_count_bins(const vox_segment *d_segs, int64_t n, vox_dims dims, v
  * anything. Arguments as for vox_generate.
  * After one vox_count, a list-only call (VOX_OUT_LIST32/64) and a volume-only
  * call (VOX_OUT_BITMASK) may run concurrently on two streams: the list reads
- * the scanned offsets (and takes its work from a counter before them, one for
- * each list type), the volume reads them and writes only the brick arrays that
- * follow them in the workspace, and errors are recorded first-wins.
+ * the scanned offsets, the volume reads them and writes only the brick arrays
+ * that follow them in the workspace, and errors are recorded first-wins.
  */
 vox_status vox_generate_from_scan(const vox_segment *d_segs, int64_t n, vox_dims dims,
                                   void *d_list, int64_t list_capacity, uint32_t *d_mask,

@@ -28,7 +28,6 @@ constexpr size_t kWsAlign = 256;
 constexpr int64_t kMaxDim = int64_t(1) << 21;
 constexpr int64_t kMinPerCta = 2048;          // smallest voxel range given to one CTA
 constexpr int64_t kDefaultWaitNs = 500000000;  // 0.5 s bound on every in-kernel wait
-static_assert(kListCounterOffset + 2 * sizeof(uint32_t) <= kWsAlign, "inside the ticket region");
 
 std::atomic<int64_t> g_stall_tile{-1};
 std::atomic<int64_t> g_wait_ns{kDefaultWaitNs};
@@ -427,19 +426,12 @@ vox_status launch_gen_t(const GenParams &p, cudaStream_t stream)
     }
 }
 
-// The list alone (k_list): the resident CTAs, whose warps take chunks sized on the device
-// from the total that the scan found, whatever the capacity. The counter they take them
-// from is in the workspace's ticket region, one per list type so that both may be written
-// after one scan; zero after every count + scan.
+// The list alone (k_list): a CTA for every chunk that the list may take. It has at most
+// `capacity` voxels, and none of its n segments more than `edge`: a buffer larger than
+// that costs no CTAs.
 template <typename PackT>
-uint32_t *list_counter(void *ws)
-{
-    return reinterpret_cast<uint32_t *>(static_cast<char *>(ws) + kListCounterOffset) + (sizeof(PackT) == 8 ? 1 : 0);
-}
-
-template <typename PackT>
-vox_status launch_list(const vox_segment *segs, int64_t n, void *list, int64_t capacity, void *ws, int32_t *status,
-                       cudaStream_t stream)
+vox_status launch_list(const vox_segment *segs, int64_t n, int64_t edge, void *list, int64_t capacity, void *ws,
+                       int32_t *status, cudaStream_t stream)
 {
     ListParams p;
     p.segs = reinterpret_cast<const int32_t *>(segs);
@@ -448,23 +440,13 @@ vox_status launch_list(const vox_segment *segs, int64_t n, void *list, int64_t c
     p.list = list;
     p.capacity = capacity;
     p.status = status;
-    p.counter = list_counter<PackT>(ws);
     auto kernel = k_list<PackT>;
-    const int grid = grid_ctas(reinterpret_cast<const void *>(kernel), kListThreads, 0);
-    if (grid <= 0) return VOX_ERR_CUDA;
-    kernel<<<static_cast<unsigned>(grid), kListThreads, 0, stream>>>(p);
+    p.resident = grid_ctas(reinterpret_cast<const void *>(kernel), kListThreads, 0);
+    if (p.resident <= 0) return VOX_ERR_CUDA;
+    const int64_t most = n < capacity / edge ? n * edge : capacity, round = list_round(p.resident);
+    const int64_t rounds = std::min(kListRounds, std::max<int64_t>(1, (most - 1) / round + 1));
+    kernel<<<static_cast<unsigned>(p.resident * rounds), kListThreads, 0, stream>>>(p);
     return cudaGetLastError() == cudaSuccess ? VOX_OK : VOX_ERR_CUDA;
-}
-
-// The list's counter zeroed for a list that does not follow a count + scan in its call,
-// where the capacity allows more than one chunk per warp (else no warp takes a second).
-template <typename PackT>
-vox_status reset_list_counter(int64_t capacity, void *ws, cudaStream_t stream)
-{
-    const int grid = grid_ctas(reinterpret_cast<const void *>(k_list<PackT>), kListThreads, 0);
-    if (grid <= 0) return VOX_ERR_CUDA;
-    if (capacity / kListChunkMax < static_cast<int64_t>(grid) * kListWarps) return VOX_OK;
-    return cudaMemsetAsync(list_counter<PackT>(ws), 0, sizeof(uint32_t), stream) == cudaSuccess ? VOX_OK : VOX_ERR_CUDA;
 }
 
 vox_status launch_generate(const vox_segment *segs, int64_t n, vox_dims dims, void *list, int64_t capacity,
@@ -498,8 +480,9 @@ vox_status launch_generate(const vox_segment *segs, int64_t n, vox_dims dims, vo
     const bool lin64 = scene_of != nullptr || volume_bits(dims) > (uint64_t(1) << 32);
     const bool bm = flags & VOX_OUT_BITMASK;
     if (!bm) {  // a list alone
-        if (flags & VOX_OUT_LIST32) return launch_list<uint32_t>(segs, n, list, capacity, ws, status, stream);
-        return launch_list<uint64_t>(segs, n, list, capacity, ws, status, stream);
+        const int64_t edge = scene_of != nullptr ? kMaxDim : std::max(dims.w, std::max(dims.h, dims.d));
+        if (flags & VOX_OUT_LIST32) return launch_list<uint32_t>(segs, n, edge, list, capacity, ws, status, stream);
+        return launch_list<uint64_t>(segs, n, edge, list, capacity, ws, status, stream);
     }
     if (flags & VOX_OUT_LIST32) return launch_gen_t<kOutList32 | kOutMask, false>(p, stream);
     if (flags & VOX_OUT_LIST64)
@@ -1134,13 +1117,8 @@ vox_status vox_generate_from_scan(const vox_segment *d_segs, int64_t n, vox_dims
     if (vox_status e = check_generate_args(d_segs, n, dims, d_list, list_capacity, d_mask, flags, d_ws, ws_bytes,
                                            d_status))
         return e;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (flags & VOX_OUT_LIST32) {
-        if (vox_status e = reset_list_counter<uint32_t>(list_capacity, d_ws, s)) return e;
-    } else if (flags & VOX_OUT_LIST64) {
-        if (vox_status e = reset_list_counter<uint64_t>(list_capacity, d_ws, s)) return e;
-    }
-    return launch_outputs(d_segs, n, dims, d_list, list_capacity, d_mask, flags, d_ws, ws_bytes, d_status, s);
+    return launch_outputs(d_segs, n, dims, d_list, list_capacity, d_mask, flags, d_ws, ws_bytes, d_status,
+                          static_cast<cudaStream_t>(stream));
 }
 
 size_t vox_workspace_size_batched(int64_t n_total, int32_t n_scenes)

@@ -28,10 +28,6 @@
 
 namespace vox {
 
-// Bytes from the scan's ticket to the chunk counters of the lists (k_list): one per list
-// type, zeroed with the ticket, or by k_scan_small.
-constexpr size_t kListCounterOffset = 128;
-
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 8;
 constexpr int kScanTile = kScanThreads * kScanItems;  // segments per scan tile
@@ -252,7 +248,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(ScanParams p)
 }
 
 // The same for a few segments, by one CTA: no tile descriptors, so nothing has to be
-// zeroed before it, and it resets the status word and the lists' counters itself. What bounds a call on so few
+// zeroed before it, and it resets the status word itself. What bounds a call on so few
 // segments is the number of operations on the stream (about 2 us each): the two memsets
 // go. Calls in a row, us: one segment of 10^5 voxels 14.8 -> 12.3 (host-bound), 2049
 // segments 17.6 -> 12.3, 4096 in 256^3 with the volume 24.4 -> 22.5. Each thread takes
@@ -269,10 +265,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_scan_small(ScanParams p)
     const int t = threadIdx.x;
     const int lane = t & 31;
     const int warp = t >> 5;
-    if (t == 0) {
-        *p.status = 0;
-        p.ticket[kListCounterOffset / 4] = p.ticket[kListCounterOffset / 4 + 1] = 0;
-    }
+    if (t == 0) *p.status = 0;
     __syncthreads();  // before any thread reports an error
     const int64_t s0 = t * kSmallItems;
     bool bad = false;

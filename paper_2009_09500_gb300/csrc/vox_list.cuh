@@ -26,13 +26,12 @@
 // carry recurrence into a shared stage (long segments) and 32-voxel thread runs with a
 // transposed stage (the rest); in the middle, rows whose lanes read a segment by eight
 // 4-byte loads, start and step apart, and pack by shifts and masks:
-//   4M log-uniform segments in 4096^3, 64-bit, 2.07e9 voxels   2720 -> 2308 -> 2327 us
-//   1024 segments, 10^9 voxels, 64-bit                         1090 -> 1048 -> 1056 us
+//   4M log-uniform segments in 4096^3, 64-bit, 2.07e9 voxels   2720 -> 2301 -> 2307 us
+//   1024 segments, 10^9 voxels, 64-bit                         1090 -> 1048 -> 1048 us
 //   1M log-uniform segments in 1000^3, 64-bit, 1.5e8 voxels     301 ->  216 ->  208 us
 //   300,000 uniform segments in 256^3, 32-bit, 4.2e7 voxels      76 ->   52 ->   43 us
 //   1M segments of 64 voxels, 32-bit, 6.7e7 voxels               78 ->   75 ->   63 us
-// (the last: 66 us by 64-voxel thread runs, which a tuning could ask for; the second step of
-// the first two lies in the order of the chunks, see k_list)
+// (the last: 66 us by 64-voxel thread runs, which a tuning could ask for)
 #pragma once
 
 #include <cstdint>
@@ -48,13 +47,15 @@ constexpr int kListWarps = 8;                  // warps per CTA
 constexpr int kListThreads = 32 * kListWarps;
 constexpr int kListCtas = 4;                   // CTAs per SM
 constexpr int kListWin = 32;                   // segments per staged window, one per lane
-// The list is cut into chunks of consecutive voxels: as many per resident warp as keep a
-// chunk within kListChunkMax, from the total that the scan found (never from the caller's
-// capacity). A warp's first chunk goes by its index, further ones by a counter, so the
-// warps at work at any moment write one front of the list (see the figures at k_list).
+// The list is cut into chunks of consecutive voxels, one per warp, as many as keep a chunk
+// within kListChunkMax, from the total that the scan found. The grid holds a CTA for every
+// chunk that the capacity allows (launch_list); CTAs beyond the total leave at once (0.3 ns
+// each). The CTAs beyond the resident ones start in order as others end, so the warps at
+// work at any moment write one front of the list (see the figures at k_list).
 constexpr int kListChunkUnit = 128;            // chunks are multiples of a row
 constexpr int kListChunkMin = 256;             // voxels per warp at least
-constexpr int kListChunkMax = 6144;            // and at most
+constexpr int kListChunkMax = 6144;            // and at most, for up to kListRounds chunks per
+constexpr int64_t kListRounds = 256;           // resident warp (7.6e9 voxels; then longer ones)
 
 struct ListParams {
     const int32_t *segs;     // [n][6]
@@ -63,8 +64,7 @@ struct ListParams {
     void *list;              // uint32 or uint64 list, 16-byte aligned
     int64_t capacity;
     int32_t *status;
-    uint32_t *counter;       // chunks taken beyond the warps' first (workspace; zero before
-                             // the launch where the total may take more than one per warp)
+    int32_t resident;        // CTAs at work at a time; the grid is a multiple of it
 };
 
 // Fixed-point words of a list type: F fraction bits, integer parts on top. Packing is a
@@ -96,13 +96,23 @@ struct ListFix<uint64_t> {
     }
 };
 
-// Voxels per chunk of a list of V voxels written by n_warps warps.
-__host__ __device__ inline int32_t list_chunk(int64_t V, int64_t n_warps)
+// Voxels that the resident CTAs' warps write with one chunk of at most kListChunkMax each.
+__host__ __device__ inline int64_t list_round(int32_t resident)
 {
-    const int64_t round = n_warps * kListChunkMax;  // voxels of one chunk per warp at most
-    const int64_t chunks = V <= round ? n_warps : n_warps * ((V + round - 1) / round);
+    return static_cast<int64_t>(resident) * (kListWarps * kListChunkMax);
+}
+
+// Voxels per chunk of a list of V voxels, by a grid of grid_rounds times the resident CTAs.
+__host__ __device__ inline int64_t list_chunk(int64_t V, int32_t resident, int64_t grid_rounds)
+{
+    const int64_t round = list_round(resident);
+    int64_t chunks = static_cast<int64_t>(resident) * kListWarps;
+    if (V > round) {
+        const int64_t rounds = (V + round - 1) / round;
+        chunks *= rounds < grid_rounds ? rounds : grid_rounds;
+    }
     const int64_t per = ((V + chunks - 1) / chunks + kListChunkUnit - 1) & ~int64_t(kListChunkUnit - 1);
-    return static_cast<int32_t>(per > kListChunkMin ? per : int64_t(kListChunkMin));
+    return per > kListChunkMin ? per : int64_t(kListChunkMin);
 }
 
 // A segment of the window: coordinates X = C + p T at position p of the chunk (the
@@ -190,15 +200,18 @@ __device__ __forceinline__ int4 list_quad(const uint64_t (&v)[2])
                      static_cast<int>(v[1] >> 32));
 }
 
-// Chunks in list order, each written front to back by one warp. What the order is worth:
-// with persistent warps taking every n_warps-th chunk the warps drift apart, and 2.07e9
-// 64-bit voxels take 2785 us; with chunks from a counter the writes stay one front and
-// take 2335 us (7.1 TB/s), whatever the list's capacity. (One chunk per warp of a grid sized
-// from the capacity, its CTAs started in order: 2308 us with a capacity of V, but 2552
-// with 3 V and 7016 with 16 V, whose chunks are of 384 voxels.) Chunks of 8192 / 12288
-// voxels at most: 2353 / 2451 us; 2048: 3416 us (the search per chunk). Rows collected in
-// shared memory and stored by 4 KB bulk copies: 2421 us, and 88 instead of 76 us on
+// One chunk per warp, written front to back. What the chunks' order is worth: with
+// persistent warps taking every n_warps-th chunk the warps drift apart, and 2.07e9
+// 64-bit voxels take 2785 us; with CTAs started in order the writes stay one front and
+// take 2308 us (7.2 TB/s), with chunks from a counter 2350 (10^9 voxels in 1024 segments
+// 1053 and 1064, 2.7e8 32-bit voxels in segments of 700 171 and 187). Chunks of 8192 /
+// 12288 voxels at most: 2353 / 2451 us; 2048: 3416 us (the search per chunk). Rows collected
+// in shared memory and stored by 4 KB bulk copies: 2421 us, and 88 instead of 76 us on
 // 64-voxel segments.
+// A capacity of 1, 3, 16 times the total, and no bound: 4M log-uniform segments 2312, 2342,
+// 2359, 2359 us; 10^9 voxels in 1024 segments 1051, 1055, 1055, 1055; 300,000 log-uniform
+// 117 each. (With chunks cut from the capacity: 2308, 2552, 7016; 1053, 1326, 6476; 117,
+// 122, 281.)
 template <typename PackT>
 __global__ void __launch_bounds__(kListThreads, kListCtas) k_list(ListParams p)
 {
@@ -206,34 +219,35 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_list(ListParams p)
     constexpr int kVox = 16 / sizeof(PackT);  // consecutive voxels per lane and row: one 16-byte store
     constexpr int kRow = 32 * kVox;
     __shared__ ListWarpSmem<PackT> s_win[kListWarps];
-    __shared__ int32_t s_go, s_chunk;
-    __shared__ int64_t s_V;
+    __shared__ int32_t s_go;
+    __shared__ int64_t s_chunk;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     ListWarpSmem<PackT> &sm = s_win[warp];
 
+    // the CTAs beyond the list: whole rounds of resident CTAs that it does not reach
+    const int64_t V = __ldg(p.offsets + p.n);
+    const uint32_t rounds_before = blockIdx.x / static_cast<uint32_t>(p.resident);
+    if (rounds_before > 0 && rounds_before * list_round(p.resident) >= V) return;
+
     // prologue decided by one thread so that the whole CTA agrees
     if (threadIdx.x == 0) {
         int32_t go = ld_volatile_i32(p.status) == 0;  // an earlier error: write nothing
-        const int64_t V = __ldg(p.offsets + p.n);
         if (go && V > p.capacity) {
             set_status(p.status, kStCapacity);
             go = 0;
         }
         s_go = go;
-        s_V = V;
-        s_chunk = list_chunk(V, static_cast<int64_t>(gridDim.x) * kListWarps);
+        s_chunk = list_chunk(V, p.resident, gridDim.x / static_cast<uint32_t>(p.resident));
     }
     __syncthreads();
     if (!s_go) return;
-    const int64_t V = s_V;
-    const int32_t chunk = s_chunk;
+    const int64_t chunk = s_chunk;
     PackT *const list = static_cast<PackT *>(p.list);
-    const uint32_t n_warps = gridDim.x * kListWarps;
     const uint32_t lt_mask = (1u << lane) - 1u;  // the lanes below
 
-    int64_t g0 = static_cast<int64_t>(blockIdx.x * kListWarps + warp) * chunk;
-    while (g0 < V) {
+    const int64_t g0 = (static_cast<int64_t>(blockIdx.x) * kListWarps + warp) * chunk;
+    if (g0 < V) {
         const int32_t len = static_cast<int32_t>(min64(chunk, V - g0));
         PackT *const out = list + g0;
         int64_t s = warp_find_segment(p.offsets, p.n, g0, lane);
@@ -363,10 +377,6 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_list(ListParams p)
             }
             s += j;
         }
-        if (static_cast<int64_t>(n_warps) * chunk >= V) break;
-        uint32_t next = 0;
-        if (lane == 0) next = atomicAdd(p.counter, 1u);
-        g0 = (static_cast<int64_t>(n_warps) + __shfl_sync(0xffffffffu, next, 0)) * chunk;
     }
 }
 
