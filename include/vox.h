@@ -446,8 +446,9 @@ vox_status vox_generate_noalloc(const vox_segment *d_segs, int64_t n, vox_dims d
  *                 alone also merged across the warp: at every step the lanes
  *                 holding equal words (__match_any_sync) OR their bits together
  *                 (__reduce_or_sync) and one lane issues the reduction)
- *   ctas_per_sm   persistent CTAs per SM for the list, atomic and brick kernels
- *                 (0 = the occupancy maximum; larger values are capped there)
+ *   ctas_per_sm   persistent CTAs per SM for the atomic and brick kernels, and the
+ *                 unit in which a list's grid is sized (0 = the occupancy maximum;
+ *                 larger values are capped there)
  *   list_runs     0, 1 or 2 (other values are 0): no effect. A list alone (no
  *                 volume in the same launch, or the volume by bricks) has one
  *                 kernel, whatever the segment lengths
