@@ -66,32 +66,15 @@ struct BrickGeom {
     int64_t n_slots;    // n_bricks * kPieceClasses * reps
 };
 
-// Pieces are at most kPieceMaxLen steps long: a longer run in one brick is cut
-// into parts of kPieceMaxLen (the last one shorter), so that no lane of the
-// brick kernel walks a long piece while the rest of its CTA waits.
-constexpr int32_t kPieceMaxLen = 64;
-
-// Half octaves of the piece length.
-constexpr int32_t piece_class(int32_t len)
-{
-    int32_t oct = 0;
-    while ((len >> oct) > 1) ++oct;
-    return 2 * oct + (oct > 0 ? (len >> (oct - 1)) & 1 : 0);
-}
-constexpr int kPieceClasses = piece_class(kPieceMaxLen) + 1;
-static_assert(kPieceClasses == 13, "no slot for lengths that no piece has");
-
+constexpr int kPieceClasses = 22;  // half octaves of the piece length (<= 1024)
 constexpr int64_t kMaxBricks = int64_t(1) << 26;
 
 // Counter replicas per (brick, class): a brick's counters are updated once per piece in
 // it, and updates of one address go one after another, so few bricks get more of them.
 // Binning of 48 scenes (1.17 M segments, 1,623 bricks in all), one counter per (brick,
 // class): 128 + 110 us (scatter, count), eight: 104 + 62 us.
-// More of them cost the slot scan what the binning gains (count + scatter + scan, us, with
-// 32 instead of 8): 1M 64-voxel segments in 1,024 bricks 28 + 48 + 5 -> 28 + 50 + 10, 3,000
-// segments there 20 + 43 + 5 -> 20 + 43 + 9, 300,000 log-uniform in 8,192 bricks 29 + 56 + 13
-// -> 29 + 57 + 26; only many segments a brick gain (48 scenes 68 + 100 + 6 -> 45 + 95 + 10).
-// Eight instead of one in 65,536 bricks: scatter 1098 -> 2475.
+// More of them cost the slot scan what the counting gains (48 scenes with 32: 46 instead
+// of 60 us of counting, 15 instead of 7 us of scanning).
 constexpr int32_t kBricks32Replicas = 512;
 constexpr int32_t kBricks8Replicas = 32768;
 
@@ -334,6 +317,11 @@ struct PieceWalker {
         return true;
     }
 };
+
+// Pieces are at most kPieceMaxLen steps long: a longer run in one brick is cut
+// into parts of kPieceMaxLen (the last one shorter), so that no lane of the
+// brick kernel walks a long piece while the rest of its CTA waits.
+constexpr int32_t kPieceMaxLen = 64;
 
 // piece = segment (32 bits) | first step (22 bits) | length - 1 (10 bits)
 __device__ __forceinline__ uint64_t pack_piece(uint32_t seg, int32_t k_lo, int32_t len)

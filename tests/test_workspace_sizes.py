@@ -32,11 +32,3 @@ def test_workspace_serves_every_smaller_volume(size, n):
 def test_batched_workspace_serves_every_smaller_batch(n_scenes):
     sizes = [vox.vox_workspace_size_batched_volume(5000, n_scenes, nb, 100) for nb in BRICKS]
     assert sizes == sorted(sizes)
-
-
-def test_no_counters_for_lengths_that_no_piece_has():
-    """A brick has a counter, an offset and a cursor (20 bytes) per replica and length
-    class; pieces are at most 64 steps long: 13 half octaves. (512 bricks against 256.)"""
-    size = lambda nb: vox.vox_workspace_size_volume(1, (256, 64 * nb, 64), 1)
-    per_brick = (size(512) - size(256)) / 256
-    assert per_brick == pytest.approx(13 * 32 * 20, rel=0.01)
