@@ -71,10 +71,10 @@ class ServeRequest:
     @property
     def device_bytes(self) -> int:
         """Volume + segments + workspace share of this request: scan, scene map, 32-byte
-        slopes, brick pieces, the slot counters of its bricks (20 bytes for each of 13
+        slopes, brick pieces, the slot counters of its bricks (20 bytes for each of 22
         length classes and at most 32 replicas) and what a batch has once."""
         return (self.mask_bytes + 24 * self.n + (16 + 32) * self.n + 8 * self.piece_capacity
-                + 13 * 32 * 21 * self.bricks + (1 << 15))
+                + 22 * 32 * 21 * self.bricks + (1 << 15))
 
     @property
     def latency_ms(self) -> float:
