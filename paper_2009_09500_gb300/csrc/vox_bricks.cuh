@@ -421,11 +421,11 @@ __device__ __forceinline__ const BrickGeom *segment_geom(const BinParams &p, int
 // four: 48 uneven scenes 110 against 100 us, 5 scenes of 1.3 M segments 241 against 203, 1M
 // 64-voxel segments 51 against 49, log-uniform 3M 859 against 839; 4M with one 1191). It
 // counts with two up to 2^20 segments and with four beyond (two against four, us):
-//   log-uniform, 2048^3   0.7M 60 : 67,  1.1M 91 : 92,  1.3M 105 : 98,  2.5M 195 : 178,  5M 383 : 340
-//   64 voxels, 1024^3     0.7M 22 : 25,  1.1M 30 : 33,  1.3M  30 : 31,  2.5M  54 :  55,  5M 108 : 107
-//   uniform, 512^3        0.7M 64 : 68,  1.1M 86 : 85,  1.3M 147 : 153, 2.5M 210 : 209,  5M 503 : 504
-//   five served scenes    1.3M 203 : 202, 1.7M 148 : 144, 296 : 270 and 337 : 326, 2.2M 265 : 239
-//   60, 70, 90, 110, 256 uneven scenes  60 : 64, 88 : 76, 87 : 91, 123 : 116, 240 : 231
+//   log-uniform, 2048^3   0.7M 61 : 65,  1.1M  91 :  92,  1.3M 106 :  97,  2.5M 195 : 180,  5M 384 : 342
+//   64 voxels, 1024^3     0.7M 22 : 25,  1.1M  30 :  32,  1.3M  31 :  31,  2.5M  54 :  54,  5M 108 : 107
+//   uniform, 512^3        0.7M 60 : 64,  1.1M 113 : 114,  1.3M 120 : 122,  2.5M 249 : 248,  5M 475 : 478
+//   five served scenes    1.3M 156 : 159,  1.7M 139 : 139, 228 : 210, 232 : 214 and 212 : 194,  2.2M 252 : 240
+//   40, 60, 80, 110, 256 uneven scenes   40 : 41,  59 : 60,  76 : 82,  107 : 104,  218 : 207
 // A lane per piece, its step and brick found by fixed-point slopes, takes about 300
 // instructions a piece (779 + 1128 us on the first).
 constexpr int kBinThreads = 256;
