@@ -688,7 +688,7 @@ __device__ __forceinline__ void find_hot(const BinParams &p)
 // Pieces written into their slots (persistent grid), and the slope table. p.G.n_slots: the number of
 // slots (all scenes' when batched). Bound by the latency of the returning atomics:
 // slot reservations of two pieces of a lane are in flight together before their
-// stores (4M log-uniform segments: 1075 us; one: 1136; four, or one held while the walk
+// stores (4M log-uniform segments: 1134 us; one: 1198; four, or one held while the walk
 // goes on: 9 to 10 % more). The first of the two waits in shared memory: in registers the
 // batched instance spills (serve-sized batches of five scenes 219 -> 206 us, 48 uneven
 // scenes 103 -> 98).

@@ -24,6 +24,7 @@ def record(tmp_path, monkeypatch):
 
 
 @pytest.mark.parametrize("tuning,found", [((0, 0, 0, 0), True), ((32, 0, 0, 0), True), ((64, 0, 0, 1), True),
+                                          ((32, 0, 4, 2), True),
                                           ((32, 0, 2, 0), False), ((32, 1, 0, 0), False)])
 def test_record_is_found_under_equal_launches(record, tuning, found):
     vox.vox_set_tuning(*tuning)
