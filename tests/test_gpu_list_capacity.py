@@ -21,8 +21,8 @@ def _scan(w):
 
 @pytest.mark.parametrize("bits", [32, 64])
 def test_large_capacities_give_the_same_list(bits):
-    """More than one chunk per warp (5e7 voxels), and far less than one; the counter of
-    the chunks is reset for every list of a scan, whatever the workspace held."""
+    """More than one chunk per resident warp (5e7 voxels), and far less than one; several
+    lists of one scan."""
     O = get_oracle()
     rng = np.random.default_rng(bits)
     for n, top in ((98_000, 1024), (300, 200)):
